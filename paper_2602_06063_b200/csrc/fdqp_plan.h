@@ -31,8 +31,8 @@ constexpr int kPlaneRecBytes = 64, kPlaneSumBytes = 32;
 //     then 64 bytes per token: the units of the eight tiles times 65536, and the units;
 //     then 128 bytes: the sums of x as a B fragment [8 tiles][8 columns], columns 4 token + {0, 1, 2} = its three bf16
 //     parts (MXFP4: instead 16 bytes per (t, token), the four planes' MMA start values).
-//   M >= 3: 64 bytes per (t, token), the bf16 activations in MMA fragment order; then 2 x 256 bytes: the three parts of
-//     the sums of x of four tiles each as a B fragment [4 x 3 parts, 4 zeros][8 tokens] (MXFP4: none).
+//   M >= 3: 64 bytes per (t, token), the bf16 activations in MMA fragment order; then 512 bytes: the sums of x as B
+//     fragments [8 tiles][8 tokens], 16 bytes per lane: its word of the first, second and third parts (MXFP4: none).
 #ifdef __CUDACC__
 __host__ __device__
 #endif

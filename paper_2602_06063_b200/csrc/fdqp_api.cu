@@ -544,7 +544,7 @@ namespace {
 // inside the GEMV kernel's activation preparation when that runs in-kernel on the whole row, else by a kernel of its own.
 fdqp_status run_impl(fdqp_ctx* ctx, const void* x_bf16, const void* gamma_bf16, float eps, const void* W_q4nx, void* out,
                      int epi, int64_t M, int64_t K, int64_t N, void* cuda_stream, int fmt = kFmtQ4nx,
-                     const void* residual_bf16 = nullptr, void* h_out_bf16 = nullptr) {
+                     const void* residual_bf16 = nullptr, void* h_out_bf16 = nullptr, bool x_once = false) {
     if (!ctx || !x_bf16 || !W_q4nx || !out) return FDQP_ERR_ARG;
     if ((residual_bf16 || h_out_bf16) && !gamma_bf16) return FDQP_ERR_ARG;
     if (h_out_bf16 && !residual_bf16) return FDQP_ERR_ARG;
@@ -577,7 +577,7 @@ fdqp_status run_impl(fdqp_ctx* ctx, const void* x_bf16, const void* gamma_bf16, 
     GemvPlan& plan = call.plan;
     const bool tensor = call.tensor, one_gemv = !tensor && M <= kMaxTokens && ctx->p_path != 1;
     if (one_gemv && !call.gemv) return FDQP_ERR_SIZE;
-    if (one_gemv && ctx->p_prep >= 0) plan.prep_inline = ctx->p_prep != 0;  // (fdqp_run_host sets it for one call)
+    if (one_gemv && x_once) plan.prep_inline = 0;  // (in this call's copy of the plan)
     bool fuse_norm = false, prepared = false;
     if (gamma) {
         // fused when the call is one GEMV launch that prepares the whole row of x inside every CTA
@@ -754,10 +754,8 @@ extern "C" fdqp_status fdqp_run_host_async(fdqp_ctx* ctx, const void* x_host_bf1
         else
             cudaGetLastError();
     }
-    const int64_t saved_prep = ctx->p_prep;
-    if (direct_x) ctx->p_prep = 0;  // x is read once, by the preparation kernel
-    st = fdqp_run(ctx, x_dev, W_q4nx, y_dev, M, K, N, cuda_stream);
-    ctx->p_prep = saved_prep;
+    // (direct_x: x is read once, by the preparation kernel)
+    st = run_impl(ctx, x_dev, nullptr, 0.f, W_q4nx, y_dev, kEpiNone, M, K, N, cuda_stream, kFmtQ4nx, nullptr, nullptr, direct_x);
     if (st != FDQP_OK) return st;
     if (y_dev == ctx->y_stage && (e = cudaMemcpyAsync(y_host, ctx->y_stage, (size_t)M * N * 4, cudaMemcpyDeviceToHost, stream)))
         return cuda_fail(ctx, e, "y copy");

@@ -825,10 +825,9 @@ extern "C" const char* fdqp_last_cuda_error(fdqp_ctx* ctx) { return ctx ? ctx->l
 extern "C" fdqp_status fdqp_set_param(fdqp_ctx* ctx, const char* key, int64_t value) {
     if (!ctx || !key) return FDQP_ERR_ARG;
     const int64_t v = value < 0 ? -1 : value;
-    {
-        std::lock_guard<std::mutex> lock(ctx->dispatch_mutex);
-        for (int i = 0; i < fdqp_ctx::kDispatchSlots; ++i) ctx->dispatch[i].M = 0;
-    }
+    // Held until the value is stored: a dispatch that another thread makes meanwhile would be kept with the old one.
+    std::lock_guard<std::mutex> lock(ctx->dispatch_mutex);
+    for (int i = 0; i < fdqp_ctx::kDispatchSlots; ++i) ctx->dispatch[i].M = 0;
     if (!std::strcmp(key, "path")) {
         if (v > 3) return FDQP_ERR_ARG;
         ctx->p_path = v;

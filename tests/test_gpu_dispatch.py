@@ -1,4 +1,8 @@
 """The table of kept dispatches: what a call launches and returns depends on its sizes and the parameters alone."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -8,6 +12,7 @@ import synthgen
 from gpu_common import Case
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _calls(ctx, case, gamma):
@@ -47,3 +52,59 @@ def test_a_host_call_leaves_no_trace_in_device_calls(K, N, M):
     for (launches, y), (launches_after, y_after) in zip(*results):
         assert launches_after == launches
         assert np.array_equal(y_after, y)
+
+
+# One thread calls fdqp_run over and over; the other sets "prep_inline", waits until the first is between calls, and counts
+# the launches of a call of its own.  (In Python the interpreter lock would keep the two apart.)
+STRESS = r"""
+#include <atomic>
+#include <thread>
+#include "fdqp.h"
+extern "C" int64_t stress(fdqp_ctx* ctx, const void* x, const void* W, float* y, int64_t K, int64_t N, void* stream, int64_t rounds) {
+    std::atomic<int> go{0}, busy{0}, stop{0};
+    std::thread other([&] {
+        while (!stop) {
+            busy = 1;
+            if (go) fdqp_run(ctx, x, W, y, 1, K, N, stream);
+            busy = 0;
+        }
+    });
+    int64_t stale = 0;
+    for (int64_t i = 0; i < rounds; ++i) {
+        go = 1;
+        for (volatile int spin = 0; spin < 500 + (int)(i % 97) * 100; ++spin) {}
+        fdqp_set_param(ctx, "prep_inline", i & 1);
+        go = 0;
+        while (busy) {}
+        const int64_t before = fdqp_launch_count(ctx);
+        fdqp_run(ctx, x, W, y, 1, K, N, stream);
+        stale += fdqp_launch_count(ctx) - before != (i & 1 ? 1 : 2);
+    }
+    stop = 1;
+    other.join();
+    return stale;
+}
+"""
+
+
+def test_a_parameter_takes_effect_under_a_concurrent_caller(tmp_path):
+    """From fdqp_set_param's return on every call obeys the new value, whatever another thread was calling meanwhile.  (Both
+    threads use one stream, so that the context's workspace has one user at a time on the device.)"""
+    lib = fd.load_library()
+    src, so = tmp_path / "stress.cpp", tmp_path / "libstress.so"
+    src.write_text(STRESS)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-pthread", "-I", os.path.join(ROOT, "include"), "-o", str(so), str(src),
+                    lib._name], check=True)
+    K, N = 2560, 64
+    case = Case(K, N, 1, seed=77)
+    y = torch.empty((1, N), dtype=torch.float32, device="cuda")
+    ctx = fd.fdqp_create(0, 1, K, N)
+    try:
+        fn = ctypes.CDLL(str(so)).stress
+        fn.restype, fn.argtypes = ctypes.c_int64, [ctypes.c_void_p] * 4 + [ctypes.c_int64] * 2 + [ctypes.c_void_p, ctypes.c_int64]
+        stale = fn(ctx, case.x_dev.data_ptr(), case.W_dev.data_ptr(), y.data_ptr(), K, N, torch.cuda.current_stream().cuda_stream, 5000)
+        torch.cuda.synchronize()
+        assert fd.fdqp_last_status(ctx) == 0
+    finally:
+        fd.fdqp_destroy(ctx)
+    assert stale == 0

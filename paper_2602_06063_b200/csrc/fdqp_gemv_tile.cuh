@@ -36,9 +36,10 @@ __device__ __forceinline__ int64_t cta_of(int64_t L, int64_t G, int64_t T) {
 //   xq[((T*M + tok)*4 + q)*4], and the group's sum of x at xsc[T*8 + tok].
 // `tile` is the group-tile index in x, `slot` the tile's index in the destination (global: the same; shared
 // memory: relative to the CTA's K slice).  Must be called by whole quads (the four q of a (tile, token)).
-__device__ __forceinline__ uint4 xprep_load(const uint16_t* __restrict__ x, int K, int tile, int tok, int q, bool valid) {
+// x may be what the launch before wrote while this one had already begun: a coherent load, and from L2 (each CTA reads it once).
+__device__ __forceinline__ uint4 xprep_load(const uint16_t* x, int K, int tile, int tok, int q, bool valid) {
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (valid) v = *reinterpret_cast<const uint4*>(x + (int64_t)tok * K + tile * kGroup + q * 8);
+    if (valid) v = __ldcg(reinterpret_cast<const uint4*>(x + (int64_t)tok * K + tile * kGroup + q * 8));
     return v;
 }
 

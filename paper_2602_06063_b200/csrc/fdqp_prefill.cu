@@ -971,15 +971,14 @@ __global__ void __launch_bounds__(kPfThreads, 1)
 }
 
 // Second phase of a K-split call: y = sum over slices z (ascending) of the partial results; four outputs per thread.
-__global__ void __launch_bounds__(256) fdqp_prefill_sum_kernel(const float4* __restrict__ ws, float4* __restrict__ y, int Z,
-                                                                int64_t quads) {
+__global__ void __launch_bounds__(256) fdqp_prefill_sum_kernel(const float4* ws, float4* y, int Z, int64_t quads) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the partial results
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= quads) return;
-    float4 acc = ws[i];
+    float4 acc = __ldcg(ws + i);
     for (int z = 1; z < Z; ++z) {
-        const float4 v = ws[(int64_t)z * quads + i];
+        const float4 v = __ldcg(ws + (int64_t)z * quads + i);
         acc.x += v.x;
         acc.y += v.y;
         acc.z += v.z;
@@ -989,15 +988,14 @@ __global__ void __launch_bounds__(256) fdqp_prefill_sum_kernel(const float4* __r
 }
 
 // The same for the bf16 / gated-GELU epilogues: one output value per thread, whole warps on one (token, strip).
-__global__ void __launch_bounds__(256) fdqp_prefill_sum_epi_kernel(const float* __restrict__ ws, uint16_t* __restrict__ y16,
-                                                                    int epi, int Z, int M, int N) {
+__global__ void __launch_bounds__(256) fdqp_prefill_sum_epi_kernel(const float* ws, uint16_t* y16, int epi, int Z, int M, int N) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the partial results
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t total = (int64_t)M * N;  // a multiple of 32
     if (idx >= total) return;
-    float acc = ws[idx];
-    for (int z = 1; z < Z; ++z) acc += ws[(int64_t)z * total + idx];
+    float acc = __ldcg(ws + idx);
+    for (int z = 1; z < Z; ++z) acc += __ldcg(ws + (int64_t)z * total + idx);
     const int tok = (int)(idx / N), n = (int)(idx - (int64_t)tok * N);
     store_output(nullptr, y16, epi, N, n >> 5, n & 31, tok, acc);
 }

@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kKvWarps * 32, 1) flowkv_decode_kernel(const F
 
 // out[h][i] = sum_s O_s[i] 2^(m_s - m*) / sum_s l_s 2^(m_s - m*) in a fixed order; one block per query head.
 template <int D>
-__global__ void __launch_bounds__(kKvMergeThreads) flowkv_merge_kernel(const float* __restrict__ ws, float* __restrict__ out, int splits) {
+__global__ void __launch_bounds__(kKvMergeThreads) flowkv_merge_kernel(const float* ws, float* out, int splits) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int h = blockIdx.x, i = threadIdx.x;
@@ -320,8 +320,8 @@ __global__ void __launch_bounds__(kKvMergeThreads) flowkv_merge_kernel(const flo
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
             const int s = i + 32 * k;
-            ms[k] = s < splits ? base[(size_t)s * (D + 4) + D] : -INFINITY;
-            ls[k] = s < splits ? base[(size_t)s * (D + 4) + D + 1] : 0.f;
+            ms[k] = s < splits ? __ldcg(base + (size_t)s * (D + 4) + D) : -INFINITY;
+            ls[k] = s < splits ? __ldcg(base + (size_t)s * (D + 4) + D + 1) : 0.f;
             m = fmaxf(m, ms[k]);
         }
 #pragma unroll
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kKvMergeThreads) flowkv_merge_kernel(const flo
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int s = part; s < splits; s += kParts) {
-        const float4 v = *reinterpret_cast<const float4*>(base + (size_t)s * (D + 4) + 4 * c);
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(base + (size_t)s * (D + 4) + 4 * c));
         const float f = factor[s];
         acc.x += v.x * f;
         acc.y += v.y * f;

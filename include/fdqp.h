@@ -57,6 +57,18 @@
  *   - Device work is enqueued on the caller's CUDA stream (a cudaStream_t passed
  *     as void*; NULL is the legacy default stream) and is asynchronous unless
  *     stated otherwise.
+ *   - Packed weights are read AHEAD of the stream order.  Every call that takes
+ *     them (fdqp_run*, fdqp_dequant*; not fdqp_run_noalloc) may begin while the
+ *     kernel before it on the stream is finishing, and fetches its first weights
+ *     then; activations, caches, outputs and workspace are touched only after
+ *     that kernel has completed.  Weights written by an ordinary kernel, copy or
+ *     memset on the same stream are complete by then.  Not so if the kernel
+ *     that writes them lets its dependents begin before it has ended
+ *     (griddepcontrol.launch_dependents, cudaTriggerProgrammaticLaunchCompletion),
+ *     or if such a kernel is the last one on the stream and weights are still
+ *     being written before it: wait for the weights on the host or with
+ *     cudaStreamSynchronize first, or set "launch_ahead" to 0 (fdqp_set_param),
+ *     after which every one of these calls is fully ordered behind the stream.
  *   - There is no CPU fallback: without an sm_100 device fdqp_create fails.
  */
 #ifndef FDQP_H
@@ -442,6 +454,9 @@ FDQP_API const char* fdqp_status_string(fdqp_status s);
  *   "l2_evict_first" 1 = weight copies carry an evict-first L2 hint
  *   "strip_aligned" 1 = CTA work ranges are cut at strip boundaries, 0 = equal block counts per CTA
  *   "prep_inline"   1 = every GEMV CTA prepares its slice of x itself, 0 = a preparation kernel runs first
+ *   "launch_ahead"  1 (default) = the kernels that read packed weights may begin while the launch before them is
+ *                   finishing, and fetch weights meanwhile; 0 = they begin after it has completed (for callers whose own
+ *                   kernels write weights and trigger their dependents early; see "Conventions")
  *   "chain_launch"  fdqp_run_chain: bit 0 = programmatic stream serialisation (default on), bit 1 = cooperative launch
  *   "chain_steps"   fdqp_run_chain: most steps per launch (1 .. 160, default 160)
  *   "chain_dependent" fdqp_run_chain: 0 (default) = a step with depends_on_previous begins a new launch; 1 = it stays in

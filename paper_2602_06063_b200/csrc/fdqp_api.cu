@@ -15,16 +15,15 @@
 #include "fdqp_plan.h"
 
 namespace fdqp {
-cudaError_t gemv_launch(const GemvPlan& p, cudaStream_t stream);
+cudaError_t gemv_launch(const GemvPlan& p, bool ahead, cudaStream_t stream);
 cudaError_t gemv_set_smem_limit(int bytes);
 cudaError_t splitk_sum_launch(const float* ws, float* y, uint16_t* y16, int epi, int Z, int S, int M, int N,
                               cudaStream_t stream);
 cudaError_t xprep_launch(const uint16_t* x, uint8_t* xq, int M, int K, int fmt, cudaStream_t stream);
-cudaError_t dequant_launch(const uint8_t* W, void* out, bool out_bf16, int K, int N, cudaStream_t stream);
-cudaError_t dequant_fmt_launch(int fmt, const uint8_t* W, void* out, bool out_bf16, int K, int N, cudaStream_t stream);
+cudaError_t dequant_launch(int fmt, const uint8_t* W, void* out, bool out_bf16, int K, int N, bool ahead, cudaStream_t stream);
 cudaError_t prefill_set_smem_limit();
 cudaError_t prefill_launch(const uint8_t* W, const uint16_t* x, int64_t x_row_bytes, float* y, uint16_t* y16, int epi, float* ws,
-                           int* status, int M, int K, int N, int pair, int Z, int fmt, int a_tmem, cudaStream_t stream,
+                           int* status, int M, int K, int N, int pair, int Z, int fmt, int a_tmem, bool ahead, cudaStream_t stream,
                            int* kernels_launched);
 cudaError_t rmsnorm_launch(const uint16_t* x, const uint16_t* residual, uint16_t* h_out, const uint16_t* gamma, float eps,
                            uint16_t* out, uint8_t* rec, int M, int K, cudaStream_t stream);
@@ -71,6 +70,7 @@ struct fdqp_ctx {
     int* chain_tickets = nullptr;
     int* chain_done = nullptr;
     size_t chain_ticket_cap = 0;
+    int64_t p_ahead = 1;  // kernels that read weights may begin, and read them, while the launch before them is finishing
     int64_t p_chain_launch = 1, p_chain_steps = kMaxChainSteps, p_chain_wide = 1, p_chain_dep = 0;
     int64_t p_flowkv_cluster = kFlowKvClusterPositions;  // ranges up to this many positions take the one-launch attention
     int64_t p_direct_y = 1;  // fdqp_run_host*: small results are stored straight into device-addressable host memory
@@ -610,7 +610,7 @@ fdqp_status run_impl(fdqp_ctx* ctx, const void* x_bf16, const void* gamma_bf16, 
         }
         int kernels = 0;
         if ((e = prefill_launch(W, xt, x_row_bytes, y, y16, epi, ctx->pf_ws, ctx->status_dev, (int)M, (int)K, (int)N,
-                                use_pair(ctx, M) ? 1 : 0, call.slices, fmt, call.tmem_mode, stream, &kernels)))
+                                use_pair(ctx, M) ? 1 : 0, call.slices, fmt, call.tmem_mode, ctx->p_ahead != 0, stream, &kernels)))
             return cuda_fail(ctx, e, "prefill kernel launch");
         ctx->launches += kernels;
         return FDQP_OK;
@@ -637,7 +637,7 @@ fdqp_status run_impl(fdqp_ctx* ctx, const void* x_bf16, const void* gamma_bf16, 
                 return cuda_fail(ctx, e, "x preparation launch");
             ctx->launches += 1;
         }
-        if ((e = gemv_launch(plan, stream))) return cuda_fail(ctx, e, "gemv kernel launch");
+        if ((e = gemv_launch(plan, ctx->p_ahead != 0, stream))) return cuda_fail(ctx, e, "gemv kernel launch");
         ctx->launches += 1;
         if (plan.Z > 1) {
             if ((e = splitk_sum_launch(ctx->ws_full, plan.y, plan.y16, epi, plan.Z, plan.S, mc, (int)N, stream)))
@@ -779,7 +779,7 @@ extern "C" fdqp_status fdqp_dequant(fdqp_ctx* ctx, const void* W_q4nx, void* out
     if (!aligned16(W_q4nx) || !aligned16(out)) return FDQP_ERR_ALIGN;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return FDQP_ERR_CUDA;
-    cudaError_t e = dequant_launch(static_cast<const uint8_t*>(W_q4nx), out, out_is_bf16 != 0, (int)K, (int)N,
+    cudaError_t e = dequant_launch(kFmtQ4nx, static_cast<const uint8_t*>(W_q4nx), out, out_is_bf16 != 0, (int)K, (int)N, ctx->p_ahead != 0,
                                    static_cast<cudaStream_t>(cuda_stream));
     if (e) return cuda_fail(ctx, e, "dequant kernel launch");
     ctx->launches += 1;
@@ -797,8 +797,8 @@ extern "C" fdqp_status fdqp_dequant_fmt(fdqp_ctx* ctx, int format, const void* W
     if (!aligned16(W_packed) || !aligned16(out)) return FDQP_ERR_ALIGN;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return FDQP_ERR_CUDA;
-    cudaError_t e = dequant_fmt_launch(format, static_cast<const uint8_t*>(W_packed), out, out_is_bf16 != 0, (int)K, (int)N,
-                                       static_cast<cudaStream_t>(cuda_stream));
+    cudaError_t e = dequant_launch(format, static_cast<const uint8_t*>(W_packed), out, out_is_bf16 != 0, (int)K, (int)N, ctx->p_ahead != 0,
+                                   static_cast<cudaStream_t>(cuda_stream));
     if (e) return cuda_fail(ctx, e, "dequant kernel launch");
     ctx->launches += 1;
     return FDQP_OK;
@@ -864,6 +864,9 @@ extern "C" fdqp_status fdqp_set_param(fdqp_ctx* ctx, const char* key, int64_t va
     } else if (!std::strcmp(key, "strip_aligned")) {
         if (v > 1) return FDQP_ERR_ARG;
         ctx->p_aligned = v;
+    } else if (!std::strcmp(key, "launch_ahead")) {
+        if (v > 1) return FDQP_ERR_ARG;
+        ctx->p_ahead = v < 0 ? 1 : v;
     } else if (!std::strcmp(key, "chain_launch")) {
         if (v > 3) return FDQP_ERR_ARG;
         ctx->p_chain_launch = v < 0 ? 1 : v;
@@ -1123,7 +1126,8 @@ extern "C" fdqp_status fdqp_run_chain(fdqp_ctx* ctx, const fdqp_chain_step* step
                                             kFmtQ4nx, u.residual_bf16, u.h_out_bf16);
             if (st != FDQP_OK) return st;
         } else {
-            const cudaError_t e = chain_launch(plans[a.index], grid, plan_epi[a.index] != 0, (int)ctx->p_chain_launch, stream);
+            const cudaError_t e = chain_launch(plans[a.index], grid, plan_epi[a.index] != 0,
+                                               (int)(ctx->p_ahead ? ctx->p_chain_launch : ctx->p_chain_launch & ~1), stream);
             if (e) return cuda_fail(ctx, e, "chain kernel launch");
             ctx->launches += 1;
         }
@@ -1221,7 +1225,7 @@ extern "C" fdqp_status fdqp_run_noalloc(const void* x_bf16, const void* W_q4nx, 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     // The array keeps whatever the last call left: the arrival counters must start at zero.
     if (cudaMemsetAsync(plan.tickets, 0, sizeof(int) * (size_t)plan.S, stream) != cudaSuccess) { cudaGetLastError(); return FDQP_ERR_CUDA; }
-    if (gemv_launch(plan, stream) != cudaSuccess) { cudaGetLastError(); return FDQP_ERR_CUDA; }
+    if (gemv_launch(plan, true, stream) != cudaSuccess) { cudaGetLastError(); return FDQP_ERR_CUDA; }
     return FDQP_OK;
 }
 

@@ -145,7 +145,7 @@ cudaError_t wait_selftest_launch(int* status, unsigned long long limit_ns, cudaS
 }
 
 template <int FMT>
-static cudaError_t dequant_fmt_launch_t(const uint8_t* W, void* out, bool out_bf16, int K, int N, cudaStream_t stream) {
+static cudaError_t dequant_fmt_launch_t(const uint8_t* W, void* out, bool out_bf16, int K, int N, bool ahead, cudaStream_t stream) {
     const int64_t ctas = (int64_t)((N / kStripRows + 7) / 8) * (K / kGroup);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas);
@@ -155,21 +155,17 @@ static cudaError_t dequant_fmt_launch_t(const uint8_t* W, void* out, bool out_bf
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;  // may overlap the launch before it (see the kernel)
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = ahead ? 1 : 0;
     return out_bf16 ? cudaLaunchKernelEx(&cfg, fdqp_dequant_tile_kernel<FMT, true>, W, out, K, N)
                     : cudaLaunchKernelEx(&cfg, fdqp_dequant_tile_kernel<FMT, false>, W, out, K, N);
 }
 
-cudaError_t dequant_launch(const uint8_t* W, void* out, bool out_bf16, int K, int N, cudaStream_t stream) {
-    return dequant_fmt_launch_t<kFmtQ4nx>(W, out, out_bf16, K, N, stream);
-}
-
-cudaError_t dequant_fmt_launch(int fmt, const uint8_t* W, void* out, bool out_bf16, int K, int N, cudaStream_t stream) {
+cudaError_t dequant_launch(int fmt, const uint8_t* W, void* out, bool out_bf16, int K, int N, bool ahead, cudaStream_t stream) {
     switch (fmt) {
-        case kFmtQ4nx: return dequant_launch(W, out, out_bf16, K, N, stream);
-        case kFmtG64: return dequant_fmt_launch_t<kFmtG64>(W, out, out_bf16, K, N, stream);
-        case kFmtG128: return dequant_fmt_launch_t<kFmtG128>(W, out, out_bf16, K, N, stream);
-        case kFmtMxfp4: return dequant_fmt_launch_t<kFmtMxfp4>(W, out, out_bf16, K, N, stream);
+        case kFmtQ4nx: return dequant_fmt_launch_t<kFmtQ4nx>(W, out, out_bf16, K, N, ahead, stream);
+        case kFmtG64: return dequant_fmt_launch_t<kFmtG64>(W, out, out_bf16, K, N, ahead, stream);
+        case kFmtG128: return dequant_fmt_launch_t<kFmtG128>(W, out, out_bf16, K, N, ahead, stream);
+        case kFmtMxfp4: return dequant_fmt_launch_t<kFmtMxfp4>(W, out, out_bf16, K, N, ahead, stream);
     }
     return cudaErrorInvalidValue;
 }

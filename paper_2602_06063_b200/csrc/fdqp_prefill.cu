@@ -1036,9 +1036,9 @@ cudaError_t prefill_set_smem_limit() {
     return prefill_set_smem_limit_fmt<kFmtMxfp4>();
 }
 
-// A launch that may overlap the one before it on the stream (see the kernels); cluster: CTAs per cluster (0: none).
+// ahead: a launch that may overlap the one before it on the stream (see the kernels); cluster: CTAs per cluster (0: none).
 template <typename... Params, typename... Args>
-static cudaError_t launch_chained(void (*kernel)(Params...), int64_t grid, int block, uint32_t smem, int cluster, cudaStream_t stream,
+static cudaError_t launch_chained(void (*kernel)(Params...), int64_t grid, int block, uint32_t smem, int cluster, bool ahead, cudaStream_t stream,
                                   Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -1046,34 +1046,41 @@ static cudaError_t launch_chained(void (*kernel)(Params...), int64_t grid, int b
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)cluster;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
+    int n = 0;
+    if (ahead) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    if (cluster) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = cluster ? 2 : 1;
+    cfg.numAttrs = (unsigned)n;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 template <int FMT>
 static cudaError_t prefill_launch_kernels(const CUtensorMap& map, const PrefillParams& p, int pair, int a_tmem, int M, int N,
-                                          int Z, cudaStream_t stream) {
+                                          int Z, bool ahead, cudaStream_t stream) {
     if (pair) {
         const int n_tiles = (N + 2 * kP2Rows - 1) / (2 * kP2Rows), tok_tiles = (M + kP2Toks - 1) / kP2Toks;
-        return launch_chained(fdqp_prefill_pair_kernel<FMT>, 2 * (int64_t)n_tiles * tok_tiles * Z, kPfThreads, kP2SmemBytes, 2, stream, map, p);
+        return launch_chained(fdqp_prefill_pair_kernel<FMT>, 2 * (int64_t)n_tiles * tok_tiles * Z, kPfThreads, kP2SmemBytes, 2, ahead, stream, map, p);
     }
     if (pair == 0 && M <= Pf1<128>::kToks) {  // small tiles, two CTAs per SM
         const int n_tiles = (N + 127) / 128;
         if (a_tmem == 2 && M <= 64)
-            return launch_chained(fdqp_prefill_kernel<FMT, 128, true, true>, (int64_t)n_tiles * Z, Pf1<128>::kThreads, Pf1<128>::kSmemBytesTri, 0, stream, map, p);
+            return launch_chained(fdqp_prefill_kernel<FMT, 128, true, true>, (int64_t)n_tiles * Z, Pf1<128>::kThreads, Pf1<128>::kSmemBytesTri, 0, ahead, stream, map, p);
         if (a_tmem)
-            return launch_chained(fdqp_prefill_kernel<FMT, 128, true>, (int64_t)n_tiles * Z, Pf1<128>::kThreads, Pf1<128>::kSmemBytesTmemA, 0, stream, map, p);
-        return launch_chained(fdqp_prefill_kernel<FMT, 128>, (int64_t)n_tiles * Z, Pf1<128>::kThreads, Pf1<128>::kSmemBytes, 0, stream, map, p);
+            return launch_chained(fdqp_prefill_kernel<FMT, 128, true>, (int64_t)n_tiles * Z, Pf1<128>::kThreads, Pf1<128>::kSmemBytesTmemA, 0, ahead, stream, map, p);
+        return launch_chained(fdqp_prefill_kernel<FMT, 128>, (int64_t)n_tiles * Z, Pf1<128>::kThreads, Pf1<128>::kSmemBytes, 0, ahead, stream, map, p);
     }
     const int n_tiles = (N + kPfRows - 1) / kPfRows, tok_tiles = (M + kPfToks - 1) / kPfToks;
-    return launch_chained(fdqp_prefill_kernel<FMT, 256>, (int64_t)n_tiles * tok_tiles * Z, Pf1<256>::kThreads, Pf1<256>::kSmemBytes, 0, stream, map, p);
+    return launch_chained(fdqp_prefill_kernel<FMT, 256>, (int64_t)n_tiles * tok_tiles * Z, Pf1<256>::kThreads, Pf1<256>::kSmemBytes, 0, ahead, stream, map, p);
 }
 
 // x: [M][K] bf16 row-major (device).  Returns cudaErrorNotSupported if the tensor map cannot be built.
@@ -1083,9 +1090,10 @@ static cudaError_t prefill_launch_kernels(const CUtensorMap& map, const PrefillP
 // x_row_bytes: distance between token rows of x (K * 2 for a dense [M][K] array; a multiple of 16).
 // epi: kEpiNone writes fp32 y; the other epilogues write bf16 to y16 (see fdqp_plan.h).
 // fmt: the container's format (fdqp_format.h).
+// ahead: the contraction may overlap the launch before it.
 // kernels_launched (may be null): receives 1, or 2 when the K slices needed the second kernel.
 cudaError_t prefill_launch(const uint8_t* W, const uint16_t* x, int64_t x_row_bytes, float* y, uint16_t* y16, int epi, float* ws,
-                           int* status, int M, int K, int N, int pair, int Z, int fmt, int a_tmem, cudaStream_t stream,
+                           int* status, int M, int K, int N, int pair, int Z, int fmt, int a_tmem, bool ahead, cudaStream_t stream,
                            int* kernels_launched) {
     if (kernels_launched) *kernels_launched = 0;
     EncodeTiledFn encode = encode_tiled_fn();
@@ -1119,10 +1127,10 @@ cudaError_t prefill_launch(const uint8_t* W, const uint16_t* x, int64_t x_row_by
     Z = p.Z;
     cudaError_t err;
     switch (fmt) {
-        case kFmtQ4nx: err = prefill_launch_kernels<kFmtQ4nx>(map, p, pair, a_tmem, M, N, Z, stream); break;
-        case kFmtG64: err = prefill_launch_kernels<kFmtG64>(map, p, pair, a_tmem, M, N, Z, stream); break;
-        case kFmtG128: err = prefill_launch_kernels<kFmtG128>(map, p, pair, a_tmem, M, N, Z, stream); break;
-        case kFmtMxfp4: err = prefill_launch_kernels<kFmtMxfp4>(map, p, pair, a_tmem, M, N, Z, stream); break;
+        case kFmtQ4nx: err = prefill_launch_kernels<kFmtQ4nx>(map, p, pair, a_tmem, M, N, Z, ahead, stream); break;
+        case kFmtG64: err = prefill_launch_kernels<kFmtG64>(map, p, pair, a_tmem, M, N, Z, ahead, stream); break;
+        case kFmtG128: err = prefill_launch_kernels<kFmtG128>(map, p, pair, a_tmem, M, N, Z, ahead, stream); break;
+        case kFmtMxfp4: err = prefill_launch_kernels<kFmtMxfp4>(map, p, pair, a_tmem, M, N, Z, ahead, stream); break;
         default: return cudaErrorInvalidValue;
     }
     if (err != cudaSuccess) return err;
@@ -1130,10 +1138,10 @@ cudaError_t prefill_launch(const uint8_t* W, const uint16_t* x, int64_t x_row_by
     if (Z == 1) return err;
     if (epi != kEpiNone) {
         const int64_t total = (int64_t)M * N;
-        return launch_chained(fdqp_prefill_sum_epi_kernel, (total + 255) / 256, 256, 0, 0, stream, (const float*)ws, y16, epi, Z, M, N);
+        return launch_chained(fdqp_prefill_sum_epi_kernel, (total + 255) / 256, 256, 0, 0, true, stream, (const float*)ws, y16, epi, Z, M, N);
     }
     const int64_t quads = (int64_t)M * N / 4;  // N is a multiple of 32
-    return launch_chained(fdqp_prefill_sum_kernel, (quads + 255) / 256, 256, 0, 0, stream, reinterpret_cast<const float4*>(ws),
+    return launch_chained(fdqp_prefill_sum_kernel, (quads + 255) / 256, 256, 0, 0, true, stream, reinterpret_cast<const float4*>(ws),
                           reinterpret_cast<float4*>(y), Z, quads);
 }
 

@@ -265,7 +265,10 @@ GemvShape gemv_choose(const fdqp_ctx* ctx, int M, int nbz, int64_t busiest, int 
     };
     if (ctx->p_ctas_per_sm == 2) better(8, 2, true, 8, kMinDepth);
     if (ctx->p_cw == 16) better(16, 1, false, 16, kMinDepth);
-    if (ctx->p_cw == 8) better(8, 1, true, 8, kMinDepth);
+    if (ctx->p_cw == 8) {
+        better(8, 1, true, 8, kMinDepth);
+        better(8, 1, false, 8, kMinDepth);
+    }
     if (busiest > 8 && busiest <= 12) better(12, 1, false, 12, 1);
     if (busiest >= (M > kColsMaxTokens ? kManyBlocks : kManyBlocksCols)) {
         better(16, 1, false, 16, kMinDepth);

@@ -108,3 +108,15 @@ def test_a_parameter_takes_effect_under_a_concurrent_caller(tmp_path):
     finally:
         fd.fdqp_destroy(ctx)
     assert stale == 0
+
+
+# rings of eight warps in half an SM's shared memory; only in all of it; sixteen warps' too large for it
+@pytest.mark.parametrize("K,N,M,warps,got", [(2560, 4096, 1, 8, 8), (2560, 262144, 8, 8, 8), (10240, 40960, 1, 8, 8), (2560, 4096, 1, 16, 16),
+                                             (10240, 40960, 1, 16, 16), (7168, 4096, 8, 16, 8)])
+def test_consumer_warps_are_what_was_asked_for_where_their_rings_fit(K, N, M, warps, got):
+    ctx = fd.fdqp_create(0, 8, K, N)
+    try:
+        fd.fdqp_set_param(ctx, "consumer_warps", warps)
+        assert f"fdqp_gemv_kernel<{got}," in fd.fdqp_describe(ctx, M, K, N)
+    finally:
+        fd.fdqp_destroy(ctx)

@@ -160,6 +160,68 @@ __device__ __forceinline__ bool wait_counter(const int* counter, int target, int
 
 }  // namespace
 
+// ---- flagged groups: evaluated in fp32 straight from Eq. 3 -----------------------------------------------------------
+//
+// For a group whose activations the fixed point cannot hold exactly (see xprep_item) the tensor-core path contributes
+// zero; before a consumer warp hands a strip piece to the reducer it adds the true contribution of every flagged
+// (group-tile, token) among the tiles it processed for that piece.  Lane r owns output row r of the strip and
+// accumulates x_k * w_hat(r, k) over the group's 32 inputs in k order, w_hat = fmaf(d, q, m) being the once-rounded
+// value of Eq. 3.  Error: 32 fp32 roundings relative to the partial
+// sums per group, far inside the acceptance bound whatever the activations' range; non-finite activations propagate.
+// The weights of those tiles have left the shared-memory ring by then and are read again from global memory: this
+// path is rare by construction (no group of ordinary activations is flagged) and is kept out of line and out of the
+// tile loop, which never looks at the flags.
+//
+// Geometry of a warp's share of a piece.  Processing-order position i = bl + pos0 (bl = block index inside the K
+// slice); the warp owns the positions with (i mod CB) in [j0, j0 + BPW) and, of each block, group-tile tw.
+struct ExactPiece {
+    const uint8_t* blk0;   // global address of the strip's first block of this K slice
+    int groups_total;      // K / 32
+    int b_first;           // first block of the K slice
+    int bl_lo, bl_hi;      // the piece's blocks (indices inside the slice)
+    int pos0;              // i - bl
+    int CB, j0, BPW, tw;
+    uint32_t unit0, unit_tile_stride;  // shared-memory address of the token's unit for tile 0, and bytes per tile
+    uint32_t raw0, raw_tile_stride;    // the same for the token's raw activations
+    uint32_t piece_stride;             // distance between the four 16-byte pieces of the raw activations
+};
+
+__device__ __noinline__ float piece_exact_token(const ExactPiece e, int lane) {
+    float acc = 0.f;
+    for (int bl = e.bl_lo; bl < e.bl_hi; ++bl) {
+        const int i = bl + e.pos0;
+        const int in_chunk = i % e.CB - e.j0;
+        if (in_chunk < 0 || in_chunk >= e.BPW) continue;
+        const int rest = e.groups_total - 8 * (e.b_first + bl);
+        const int jb = rest < 8 ? rest : 8;  // groups of this block (short only at the end of K)
+        if (e.tw >= jb) continue;
+        const int tile = bl * 8 + e.tw;
+        float unit;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(unit) : "r"(e.unit0 + (uint32_t)tile * e.unit_tile_stride));
+        if (unit != 0.f) continue;  // not flagged (same answer in every lane)
+        const uint8_t* blk = e.blk0 + (int64_t)bl * kBlockBytes;
+        const uint4 c = __ldg(reinterpret_cast<const uint4*>(blk + e.tw * 512 + lane * 16));
+        const uint32_t cw[4] = {c.x, c.y, c.z, c.w};
+        const int word = (e.tw * 32 + lane) * 2;
+        const float d = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(blk + 512 * jb + word)) << 16);
+        const float m = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(blk + 576 * jb + word)) << 16);
+        const uint32_t raw = e.raw0 + (uint32_t)tile * e.raw_tile_stride;
+#pragma unroll 1
+        for (int p4 = 0; p4 < 4; ++p4) {
+            uint32_t xw[4];  // (the records are 8-byte aligned)
+            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(xw[0]), "=r"(xw[1]) : "r"(raw + (uint32_t)p4 * e.piece_stride));
+            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(xw[2]), "=r"(xw[3]) : "r"(raw + (uint32_t)p4 * e.piece_stride + 8u));
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {  // byte j of code word p4: k = 8 p4 + 2j in the low nibble, k + 1 in the high one
+                const uint32_t byte = (cw[p4] >> (8 * j)) & 0xffu;
+                acc = fmaf(bf16_lo_to_f32(xw[j]), fmaf(d, (float)(byte & 15u), m), acc);
+                acc = fmaf(bf16_hi_to_f32(xw[j]), fmaf(d, (float)(byte >> 4), m), acc);
+            }
+        }
+    }
+    return acc;
+}
+
 // MODE as in the single-call kernel (1: M = 1, 3: M = 2, 2: M = 3 .. 8); BPW: blocks per consumer warp and ring stage
 // (2 or 4); EPI: built with the bf16 epilogues and the fused RMS normalisation.  Q4NX only; 16 consumer warps, a
 // producer warp, two reducer warps.
@@ -168,7 +230,6 @@ __global__ void __launch_bounds__(kThreads, 1) fdqp_chain_kernel(const __grid_co
     extern __shared__ __align__(128) uint8_t smem[];
     using MT = ModeTraits<MODE>;
     constexpr int NT = MT::kAcc;
-    constexpr int FMT = kFmtQ4nx;
     constexpr int kBPW = BPW;
     constexpr int kCB = (kCW / 8) * kBPW;   // blocks per ring stage
     constexpr uint32_t kStageBytes = kCB * kBB;
@@ -478,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1) fdqp_chain_kernel(const __grid_co
                         for (int tk = 0; tk < MT::kAccM; ++tk) {
                             ep.unit0 = xs + (uint32_t)(tk * kColsRecBytes + kColsUnitOff);
                             ep.raw0 = xs + (uint32_t)(tk * kColsRecBytes);
-                            acc_m[tk] += piece_exact_token<FMT>(ep, lane);
+                            acc_m[tk] += piece_exact_token(ep, lane);
                         }
                     }
                 }

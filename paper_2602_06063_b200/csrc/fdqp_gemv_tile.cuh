@@ -60,7 +60,7 @@ __device__ __forceinline__ uint4 add_bf16x8(uint4 a, uint4 b) {
 // is not (a value more than four million times smaller than an outlier beside it, a subnormal beside a normal
 // number), or with a non-finite element, is FLAGGED instead of rounded: its record carries unit = 0 and sum = 0, so
 // that the tensor-core path contributes exactly nothing for it, and the raw bf16 activations in k order in bytes
-// 0..63 (where the planes would be).  The chained kernel then evaluates that group in fp32 straight from Eq. 3 (piece_exact_token below).
+// 0..63 (where the planes would be).  The chained kernel then evaluates that group in fp32 straight from Eq. 3 (piece_exact_token in fdqp_chain.cu).
 template <bool SINGLE>
 __device__ __forceinline__ bool xprep_item(const uint4 v, int M, int slot, int tok, int q, bool valid,
                                            uint32_t* __restrict__ xq, float* __restrict__ xsc) {
@@ -371,89 +371,6 @@ __device__ __forceinline__ void tile_compute(const TileIn& t, float (&acc)[4][Mo
             }
         }
     }
-}
-
-// ---- flagged groups: evaluated in fp32 straight from Eq. 3 -----------------------------------------------------------
-//
-// For a group whose activations the fixed point cannot hold exactly (see xprep_item) the tensor-core path contributes
-// zero; before a consumer warp hands a strip piece to the reducer it adds the true contribution of every flagged
-// (group-tile, token) among the tiles it processed for that piece.  Lane r owns output row r of the strip and
-// accumulates x_k * w_hat(r, k) over the group's 32 inputs in k order, w_hat = fmaf(d, q, m) being the once-rounded
-// value of Eq. 3 (MXFP4: element times power-of-two scale, exact).  Error: 32 fp32 roundings relative to the partial
-// sums per group, far inside the acceptance bound whatever the activations' range; non-finite activations propagate.
-// The weights of those tiles have left the shared-memory ring by then and are read again from global memory: this
-// path is rare by construction (no group of ordinary activations is flagged) and is kept out of line and out of the
-// tile loop, which never looks at the flags.
-//
-// Geometry of a warp's share of a piece.  Processing-order position i = bl + pos0 (bl = block index inside the K
-// slice); the warp owns the positions with (i mod CB) in [j0, j0 + BPW) and, of each block, group-tile tw.
-struct ExactPiece {
-    const uint8_t* blk0;   // global address of the strip's first block of this K slice
-    int groups_total;      // K / 32
-    int b_first;           // first block of the K slice
-    int bl_lo, bl_hi;      // the piece's blocks (indices inside the slice)
-    int pos0;              // i - bl
-    int CB, j0, BPW, tw;
-    uint32_t unit0, unit_tile_stride;  // shared-memory address of the token's unit for tile 0, and bytes per tile
-    uint32_t raw0, raw_tile_stride;    // the same for the token's raw activations
-    uint32_t piece_stride;             // distance between the four 16-byte pieces of the raw activations
-};
-
-template <int FMT>
-__device__ __noinline__ float piece_exact_token(const ExactPiece e, int lane) {
-    using F = FmtTraits<FMT>;
-    float acc = 0.f;
-    for (int bl = e.bl_lo; bl < e.bl_hi; ++bl) {
-        const int i = bl + e.pos0;
-        const int in_chunk = i % e.CB - e.j0;
-        if (in_chunk < 0 || in_chunk >= e.BPW) continue;
-        const int rest = e.groups_total - 8 * (e.b_first + bl);
-        const int jb = rest < 8 ? rest : 8;  // groups of this block (short only at the end of K, Q4NX only)
-        if (e.tw >= jb) continue;
-        const int tile = bl * 8 + e.tw;
-        float unit;
-        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(unit) : "r"(e.unit0 + (uint32_t)tile * e.unit_tile_stride));
-        if (unit != 0.f) continue;  // not flagged (same answer in every lane)
-        const uint8_t* blk = e.blk0 + (int64_t)bl * F::kBlock;
-        const uint4 c = __ldg(reinterpret_cast<const uint4*>(blk + e.tw * 512 + lane * 16));
-        const uint32_t cw[4] = {c.x, c.y, c.z, c.w};
-        float d, m = 0.f;
-        if (F::kMx) {
-            // half the scale: the element table below holds twice the E2M1 value (a scale byte of 0 counts as zero)
-            d = 0.5f * __uint_as_float((uint32_t)__ldg(blk + kCodeBytes + e.tw * 32 + lane) << 23);
-        } else {
-            const int sect = FMT == kFmtQ4nx ? 512 * jb : kCodeBytes;
-            const int osect = FMT == kFmtQ4nx ? 576 * jb : (int)F::kOffSect;
-            const int word = ((e.tw >> F::kShift) * 32 + lane) * 2;
-            d = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(blk + sect + word)) << 16);
-            m = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(blk + osect + word)) << 16);
-        }
-        const uint32_t raw = e.raw0 + (uint32_t)tile * e.raw_tile_stride;
-#pragma unroll 1
-        for (int p4 = 0; p4 < 4; ++p4) {
-            uint32_t xw[4];  // (the records are 8-byte aligned)
-            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(xw[0]), "=r"(xw[1]) : "r"(raw + (uint32_t)p4 * e.piece_stride));
-            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(xw[2]), "=r"(xw[3]) : "r"(raw + (uint32_t)p4 * e.piece_stride + 8u));
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {  // byte j of code word p4: k = 8 p4 + 2j in the low nibble, k + 1 in the high one
-                const uint32_t byte = (cw[p4] >> (8 * j)) & 0xffu;
-                float w0, w1;
-                if (F::kMx) {
-                    const uint32_t q0 = byte & 15u, q1 = byte >> 4;
-                    const float v0 = (float)((0xC8643210u >> (4u * (q0 & 7u))) & 15u) * d;  // 2|value|: 0 1 2 3 4 6 8 12
-                    const float v1 = (float)((0xC8643210u >> (4u * (q1 & 7u))) & 15u) * d;
-                    w0 = (q0 & 8u) ? -v0 : v0;
-                    w1 = (q1 & 8u) ? -v1 : v1;
-                } else {
-                    w0 = fmaf(d, (float)(byte & 15u), m);
-                    w1 = fmaf(d, (float)(byte >> 4), m);
-                }
-                acc = fmaf(bf16_lo_to_f32(xw[j]), w0, acc);
-                acc = fmaf(bf16_hi_to_f32(xw[j]), w1, acc);
-            }
-        }
-    }
-    return acc;
 }
 
 // OR of a predicate over the `nthreads` threads that meet at named barrier `id` (one barrier instruction).

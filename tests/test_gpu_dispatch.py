@@ -54,6 +54,61 @@ def test_a_host_call_leaves_no_trace_in_device_calls(K, N, M):
         assert np.array_equal(y_after, y)
 
 
+def test_interleaved_shapes_keep_their_launches_and_bits():
+    """More shapes than the table has slots, plain, with epilogues, normalised and of other formats, called in shuffled orders
+    without a parameter being touched in between: each call launches and returns what it does on a context of its own."""
+    rng = np.random.default_rng(5)
+    max_M, max_K, max_N = 40, 3072, 640
+    calls = []
+    for i in range(96):
+        kind = ("run", "bf16", "norm", "fmt")[i % 4]
+        M = int(rng.choice([1, 2, 3, 4, 8, 9, 40]))
+        K = int(rng.integers(1, max_K // 256 + 1)) * 256 if kind == "fmt" else int(rng.integers(2, max_K // 32 + 1)) * 32
+        N = int(rng.integers(1, max_N // 32 + 1)) * 32
+        x = torch.from_numpy(synthgen.activations(200 + i, M, K).view(np.int16)).cuda()
+        if kind == "fmt":
+            w = synthgen.weights_fmt(300 + i, K, N, fd.FMT_MXFP4)
+            W = torch.from_numpy(fd.q4nx_pack_fmt(fd.FMT_MXFP4, w.codes, w.scales, w.offsets)).cuda()
+        else:
+            w = synthgen.weights(300 + i, K, N)
+            W = torch.from_numpy(fd.q4nx_pack(w.codes, w.scales, w.offsets)).cuda()
+        calls.append((kind, M, K, N, x, W))
+
+    def call(ctx, c):
+        kind, M, K, N, x, W = c
+        out = torch.zeros((M, N), dtype=torch.int16 if kind == "bf16" else torch.int32, device="cuda")
+        before = fd.fdqp_launch_count(ctx)
+        if kind == "run":
+            fd.fdqp_run(ctx, x, W, out, M, K, N)
+        elif kind == "bf16":
+            fd.fdqp_run_epilogue(ctx, x, W, out, fd.EPI_BF16, M, K, N)
+        elif kind == "norm":
+            fd.fdqp_run_rmsnorm_epilogue(ctx, x, x, 1e-6, W, out, fd.EPI_NONE, M, K, N)
+        else:
+            fd.fdqp_run_fmt(ctx, fd.FMT_MXFP4, x, W, out, M, K, N)
+        launches = fd.fdqp_launch_count(ctx) - before
+        torch.cuda.synchronize()
+        assert fd.fdqp_last_status(ctx) == 0
+        return launches, out
+
+    expected = []
+    for c in calls:
+        ctx = fd.fdqp_create(0, max_M, max_K, max_N)
+        try:
+            expected.append(call(ctx, c))
+        finally:
+            fd.fdqp_destroy(ctx)
+    ctx = fd.fdqp_create(0, max_M, max_K, max_N)
+    try:
+        for _ in range(3):
+            for i in rng.permutation(len(calls)):
+                launches, out = call(ctx, calls[i])
+                assert launches == expected[i][0], calls[i][:4]
+                assert torch.equal(out, expected[i][1]), calls[i][:4]
+    finally:
+        fd.fdqp_destroy(ctx)
+
+
 # One thread calls fdqp_run over and over; the other sets "prep_inline", waits until the first is between calls, and counts
 # the launches of a call of its own.  (In Python the interpreter lock would keep the two apart.)
 STRESS = r"""

@@ -178,6 +178,8 @@ NORM_CASES = [
     (2560, 2048, 1, {}, 1),                # fused into the GEMV launch
     (1152, 288, 3, {}, 1),                 # fused, three token rows, tail block
     (2560, 512, 2, {}, 2),                 # more than one item per thread: norm kernel + GEMV (which prepares in-kernel)
+    (2560, 512, 4, {}, 2),                 # three and more token rows: the norm kernel leaves the rows prepared for the GEMV launch
+    (1056, 320, 8, {}, 2),                 # the same, short last block (its absent group-tiles are prepared from zeros)
     (10240, 320, 1, {}, 3),                # too many items for in-kernel preparation: norm kernel + preparation + GEMV
     (1056, 320, 20, {"path": 2}, 6),       # norm kernel, two GEMV chunks of eight rows with their preparation, one of four without
     (1056, 320, 40, {"path": 3, "prefill_split_k": 2}, 3),  # norm kernel + tensor-core kernel (K slices) + its sum kernel

@@ -271,7 +271,7 @@ def test_batched_rows_match_single_row_calls(fresh):
 
 
 @pytest.mark.parametrize("key,values", [("split_k", [1, 2, 4, 8]), ("consumer_warps", [8, 16]), ("ctas_per_sm", [1, 2]),
-                                        ("stages", [2, 3, 7]), ("l2_evict_first", [0, 1]), ("prep_inline", [0, 1]), ("strip_aligned", [0, 1]), ("blocks_per_warp", [2, 4])])
+                                        ("stages", [2, 3, 7]), ("l2_evict_first", [0, 1]), ("prep_inline", [0, 1]), ("strip_aligned", [0, 1])])
 def test_launch_parameters_do_not_change_results(fresh, key, values):
     K, N, M = 4352, 2080, 3   # 17 blocks per strip, 65 strips: ragged against every split and grid
     case = Case(K, N, M, seed=90)

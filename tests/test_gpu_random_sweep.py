@@ -12,7 +12,7 @@ from gpu_common import ABS_TOL, REL_TOL, Case, assert_close, dev_bytes
 
 pytestmark = pytest.mark.gpu
 
-PARAMS = ("strip_aligned", "split_k", "blocks_per_warp", "path", "prefill_split_k", "prefill_pair")
+PARAMS = ("strip_aligned", "split_k", "consumer_warps", "path", "prefill_split_k", "prefill_pair")
 
 
 @pytest.fixture(scope="module")
@@ -36,7 +36,7 @@ def one_case(ctx, rng):
     if rng.random() < 0.2 and M <= 8:
         params["split_k"] = int(rng.choice([2, 4]))
     if rng.random() < 0.2:
-        params["blocks_per_warp"] = int(rng.choice([2, 4]))
+        params["consumer_warps"] = int(rng.choice([8, 16]))
     if M >= 9 and K >= 256 and rng.random() < 0.5:
         params["path"] = int(rng.choice([2, 3]))
     if M >= 9 and rng.random() < 0.3:

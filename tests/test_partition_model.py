@@ -96,3 +96,73 @@ def test_every_block_once_and_reader_matches_writers(S, nb):
         # a slot is never shared by two strips' live pieces
         edge = [p[5] for p in pieces if p[5] != "direct"]
         assert len(edge) == len(set(edge))
+
+
+# ---- a CTA's range over its warps ------------------------------------------------------------------------------------
+
+def warp_pieces(a, e, ln, warps):
+    """What the warps of a CTA do with its blocks [a, e): (warp, strip, first, past the last, where), `where` being "direct" for
+    a whole strip, "exchange" for the CTA's whole share of one it shares with other CTAs, else the warp's head or tail slot."""
+    n = e - a
+    begin = [a + n * w // warps for w in range(warps + 1)]
+    out = []
+    for w in range(warps):
+        b = begin[w]
+        while b < begin[w + 1]:
+            s = b // ln
+            u0 = s * ln
+            end = min(u0 + ln, begin[w + 1])
+            last = end == begin[w + 1]
+            if b == u0 and end == u0 + ln:
+                where = "direct"
+            elif (b == u0 or b == a) and (end == u0 + ln or end == e):
+                where = "exchange"
+            else:
+                where = "tail" if last else "head"
+            out.append((w, s, b, end, where))
+            b = end
+    return begin, out
+
+
+def combined(a, e, ln, warps, begin):
+    """What the warps add up after the last block: strip -> (the adding warp, [(warp, slot)], whole strip)."""
+    got = {}
+    for w in range(warps):
+        if begin[w] == begin[w + 1]:
+            continue
+        s = (begin[w + 1] - 1) // ln                 # the strip of the warp's last block
+        lo, hi = max(s * ln, a), min(s * ln + ln, e)
+        if begin[w + 1] < hi and lo >= begin[w]:
+            slots = [(w, "tail")]
+            for v in range(w + 1, warps):
+                if begin[v] >= hi:
+                    break
+                if begin[v] < begin[v + 1]:
+                    slots.append((v, "tail" if begin[v + 1] <= hi else "head"))
+            assert s not in got
+            got[s] = (w, slots, hi - lo == ln)
+    return got
+
+
+@pytest.mark.parametrize("warps", [4, 8, 12, 16])
+@pytest.mark.parametrize("ln", [1, 2, 3, 5, 10, 15, 42, 84])
+def test_warps_cover_a_cta_and_every_shared_strip_is_added_once(warps, ln):
+    for a in sorted({0, 1, ln - 1, ln, 2 * ln + ln // 2}):
+        for n in list(range(1, 3 * warps)) + [5 * ln, 7 * ln + 1, 105, 211, 1000]:
+            e = a + n
+            begin, pieces = warp_pieces(a, e, ln, warps)
+            assert sorted(b for _, _, lo, hi, _ in pieces for b in range(lo, hi)) == list(range(a, e))
+            shares = combined(a, e, ln, warps, begin)
+            waiting = {}
+            for w, s, lo, hi, where in pieces:
+                if where in ("head", "tail"):
+                    waiting.setdefault(s, []).append((w, where))
+                if where == "exchange":             # the one piece of the strip in this CTA
+                    assert (lo, hi) == (max(s * ln, a), min(s * ln + ln, e)) and s not in shares
+            # every piece left in a slot is added exactly once, by the strip's first warp, from the slot it was left in
+            assert {s: v[1] for s, v in shares.items()} == waiting
+            for s, (w, slots, whole) in shares.items():
+                assert whole == (s * ln >= a and s * ln + ln <= e)
+            # a warp leaves at most one piece in each of its slots: none overwrites another
+            left = [(w, where) for w, _, _, _, where in pieces if where in ("head", "tail")]
+            assert len(left) == len(set(left))

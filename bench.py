@@ -39,7 +39,7 @@ L2_BYTES = 126e6
 LAYER_COPIES = 8            # distinct weight sets resident in HBM (8 x 59 MB = 472 MB >> L2)
 NOMINAL_HBM_GBS = 8000.0
 # dram__bytes_read.sum + dram__bytes_write.sum of one LM-head launch (K=2560, N=262144, M=1) from an ncu capture
-NCU_LM_HEAD_DRAM_BYTES = 419511296 + 3408128
+NCU_LM_HEAD_DRAM_BYTES = 419496960 + 4712960
 
 
 def alg_bytes(M, K, N):

@@ -3,6 +3,12 @@
 #pragma once
 #include <stdint.h>
 
+#ifdef __CUDACC__
+#define FDQP_HD __host__ __device__
+#else
+#define FDQP_HD
+#endif
+
 namespace fdqp {
 
 constexpr int kStripRows = 32;      // output features per strip
@@ -33,10 +39,7 @@ constexpr int kPlaneRecBytes = 64, kPlaneSumBytes = 32;
 //     parts (MXFP4: instead 16 bytes per (t, token), the four planes' MMA start values).
 //   M >= 3: 64 bytes per (t, token), the bf16 activations in MMA fragment order; then 512 bytes: the sums of x as B
 //     fragments [8 tiles][8 tokens], 16 bytes per lane: its word of the first, second and third parts (MXFP4: none).
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-constexpr int gemv_rec_bytes(int M, bool mx) {
+FDQP_HD constexpr int gemv_rec_bytes(int M, bool mx) {
     return M <= kColsMaxTokens ? M * 1088 + (mx ? M * 128 : 128) : M * 512 + (mx ? 0 : 512);
 }
 constexpr int kMaxDepth = 16;       // blocks a warp's ring holds at most
@@ -111,6 +114,29 @@ struct StreamParams {
     uint32_t x_box_bytes;   // 64 k x n_inst / 2 tokens; x_steps (2 or 4) to a stage
     uint32_t smem_bytes;
 };
+
+// First unit of a pair's range, and the pair whose range holds a unit (quantum 1).
+FDQP_HD inline int st_range_begin(const StreamParams& p, int pair) {
+    return (pair * p.per_pair + (pair < p.one_more ? pair : p.one_more)) * p.quantum;
+}
+FDQP_HD inline int st_owner(const StreamParams& p, int unit) {
+    const int big = p.one_more * (p.per_pair + 1);
+    return unit < big ? unit / (p.per_pair + 1) : p.one_more + (unit - big) / p.per_pair;
+}
+
+// The barrier (0, 1: of an accumulator set; kStAccLast) that tells that segment idx of a range, its idx-th part of a tile, is in the
+// accumulators, and the number of that barrier's phase.  A wait sees a phase's parity only, so its warp has to know the phase
+// before to be complete.  Warps that read every segment of a set do.  The last segment is read by the conversion warps, which
+// where there are two sets have waited for no other one: it has a barrier of its own, used once.
+constexpr int kStAccLast = 2;
+struct StAccWait {
+    int bar;
+    uint32_t phase;
+};
+FDQP_HD inline StAccWait st_acc_wait(int acc_sets, int idx, bool last) {
+    if (last) return {kStAccLast, 0u};
+    return acc_sets == 2 ? StAccWait{idx & 1, (uint32_t)idx >> 1} : StAccWait{0, (uint32_t)idx};
+}
 
 // ---- a chain of projections in one persistent launch (fdqp_chain.cu) ---------------------------------------------
 constexpr int kMaxChainSteps = 160;  // projections one launch walks (a longer chain is cut into several launches)

@@ -155,13 +155,6 @@ struct SharedTile {
     __device__ __forceinline__ float4* slot(int r) const { return base + (2 * r + (r == p0 ? first : 0)) * slot_quads; }
 };
 
-__device__ __forceinline__ int st_range_begin(const StreamParams& p, int pair) {
-    return (pair * p.per_pair + (pair < p.one_more ? pair : p.one_more)) * p.quantum;
-}
-__device__ __forceinline__ int st_owner(const StreamParams& p, int unit) {  // (quantum 1)
-    const int big = p.one_more * (p.per_pair + 1);
-    return unit < big ? unit / (p.per_pair + 1) : p.one_more + (unit - big) / p.per_pair;
-}
 __device__ __forceinline__ SharedTile shared_tile(const StreamParams& p, int tile, int strip8, int lane) {
     SharedTile s;
     s.p0 = st_owner(p, tile * p.nb);
@@ -308,13 +301,13 @@ __device__ __forceinline__ void finish_cluster(const StreamParams& p, uint32_t e
 // this warp's strip, and stores y or, where the tile is shared, partial sums.  The last pair at a part's counter adds them; one
 // that finds all the others there before its own sums are complete leaves these where they are.
 template <bool CLUSTER>
-__device__ __forceinline__ bool st_finish(const StreamParams& p, uint32_t acc_bars, uint32_t exchange, int u0, int u1, int e, int h0, int h1) {
+__device__ __forceinline__ bool st_finish(const StreamParams& p, uint32_t acc_bars, uint32_t acc_last, uint32_t exchange, int u0, int u1, int e, int h0, int h1) {
     const int lane = threadIdx.x & 31, q = (threadIdx.x >> 5) & 3, pair = (int)(blockIdx.x >> 1);
     const uint32_t crank = cluster_ctarank();
     const int strip8 = 4 * (int)(crank & 1u) + q;
     const int tile = (e - 1) / p.nb, idx = tile - u0 / p.nb;
     const int b = p.acc_sets == 2 ? idx & 1 : 0;
-    const uint32_t parity = (uint32_t)(p.acc_sets == 2 ? idx >> 1 : idx) & 1u;
+    const StAccWait full = st_acc_wait(p.acc_sets, idx, e == u1);
     const int n_tile = tile / p.tok_tiles, tok0 = (tile - n_tile * p.tok_tiles) * p.n_inst;
     const int toks = p.M - tok0 < p.n_inst ? p.M - tok0 : p.n_inst;
     const int strip = n_tile * 8 + strip8;
@@ -332,7 +325,7 @@ __device__ __forceinline__ bool st_finish(const StreamParams& p, uint32_t acc_ba
             others = __all_sync(0xffffffffu, seen == s.p1 - s.p0);
         }
     }
-    if (!warp_wait(acc_bars + 8u * (uint32_t)b, parity, p.status)) return false;
+    if (!warp_wait(full.bar == kStAccLast ? acc_last : acc_bars + 8u * (uint32_t)b, full.phase & 1u, p.status)) return false;
     tc_fence_after();
     if (CLUSTER) {
         finish_cluster(p, exchange, acc, q, h0, crank, strip, rows, toks, lane);
@@ -398,11 +391,12 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
     const uint32_t bars = exchange + p.exchange_bytes;
     auto full_a = [&](int s) { return bars + 8u * (uint32_t)s; };                                  // CTA 0's: 16 warps
     auto empty_a = [&](int s) { return bars + 8u * (uint32_t)(4 + s); };                            // each its own, by commit
-    auto acc_full = [&](int b) { return bars + 8u * (uint32_t)(8 + b); };                           // each its own, by commit
+    auto acc_full = [&](int b) { return bars + 8u * (uint32_t)(8 + b); };                           // each its own, by commit (and acc_last)
     auto acc_empty = [&](int b) { return bars + 8u * (uint32_t)(10 + b); };                         // CTA 0's: the warps that read it
     auto full_w = [&](int s) { return bars + 8u * (uint32_t)(12 + s); };                            // each its own: 2 warps + bytes
     auto empty_w = [&](int s) { return bars + 8u * (uint32_t)(12 + kStMaxW + s); };                 // each its own: 8 warps
     const uint32_t tmem_slot = bars + 8u * (uint32_t)(12 + 2 * kStMaxW);
+    const uint32_t acc_last = tmem_slot + 8u;
     const uint32_t x_bars = tmem_slot + 16u;
     auto full_x = [&](int s) { return x_bars + 8u * (uint32_t)s; };                                 // CTA 0's: 1 + both CTAs' bytes
     auto empty_x = [&](int s) { return x_bars + 8u * (uint32_t)(p.x_stages + s); };                 // each its own, by commit
@@ -462,6 +456,7 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
         tmem_alloc2(tmem_slot, 512);
         tmem_relinquish2();
     } else if (warp == 4) {
+        if (lane == 12) mbar_init(acc_last, 1);
         if (lane < 12) mbar_init(bars + 8u * (uint32_t)lane, lane < 4 ? 16u : (lane < 10 ? 1u : (p.acc_sets == 1 ? 8u * kStParts : 8u)));
         mbar_fence_init();
     } else if (warp == 6) {
@@ -568,7 +563,7 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                             }
                         umma2_commit(used_a, pair_mask);
                         if (!p.x_resident) umma2_commit(used_x, pair_mask);
-                        if (done) umma2_commit(acc_full(b), pair_mask);
+                        if (done) umma2_commit(u + 1 == u1 ? acc_last : acc_full(b), pair_mask);
                     }
                 } else {
 #pragma unroll
@@ -595,7 +590,7 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                     }
                     if (leader) {
                         umma2_commit(used_a, pair_mask);
-                        if (done) umma2_commit(acc_full(b), pair_mask);
+                        if (done) umma2_commit(u + 1 == u1 ? acc_last : acc_full(b), pair_mask);
                     }
                 }
                 __syncwarp();
@@ -623,9 +618,10 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
     } else {
         // =============================== conversion; accumulators -> y =======================================
         // Strip (= the warp's lane quarter of tensor memory) and place i among the strip's warps: half i % 2 of every second block.
-        // (When a warp comes round, the block before its last one has been through the MMAs, which take the blocks in order: it
-        // waited for a stage of converted weights.  So with four stages of packed weights or more, and two of converted ones, no
-        // wait can mistake a stage's phase for that of two uses before.)
+        // (A wait tells a stage's phase from the next one only, not from that of two uses before.  When a warp comes round, the
+        // block a_stages before its last one has been through the MMAs, which take the blocks in order: it waited for that stage of
+        // converted weights.  So with four stages of packed weights or more, and two or three of converted ones, the use before the
+        // one that it waits for is complete.  The accumulators of a range's last segment: st_acc_wait.)
         const bool converts = warp >= 8;
         const int q = warp & 3, i = converts ? (warp - 8) >> 2 : 0, t0 = 4 * (i & 1);
         const uint32_t full0 = mapa_shared(full_a(0), leader_cta);
@@ -723,7 +719,7 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
             if (!ok) break;
             if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
             waited = true;
-            ok = st_finish<CLUSTER>(p, acc_full(0), exchange, u0, u1, seg_end, converts ? i : 0, converts ? i + 1 : kStParts);
+            ok = st_finish<CLUSTER>(p, acc_full(0), acc_last, exchange, u0, u1, seg_end, converts ? i : 0, converts ? i + 1 : kStParts);
             if (seg_end == u1) break;
             seg_end = seg_end + p.nb < u1 ? seg_end + p.nb : u1;
         }

@@ -75,6 +75,24 @@ def test_every_cut_is_exact_on_exact_inputs(ctx, K, N, M, params):
     assert np.array_equal(case.run(ctx).astype(np.float64), y_ref)
 
 
+# Three and more tiles to a pair of SMs, of one block of K (160 tiles) and of two (with five blocks to a pair a range ends in the
+# middle of a tile): the last of them is read by warps that have read none of the others.  Both numbers of stages of converted weights.
+@pytest.mark.parametrize("K,N,params", [(32, 40960, {}), (256, 40960, {}), (288, 40960, {}), (512, 47360, {"prefill_blocks": 5}), (512, 56864, {"prefill_blocks": 7})])
+@pytest.mark.parametrize("M", [17, 33, 48, 64, 100, 128])
+def test_short_tiles_in_a_row(ctx, K, N, params, M):
+    case = Case(K, N, M, seed=0, weights=exact_regime_weights(85, K, N), x=exact_regime_x(86, M, K))
+    configure(ctx, params)
+    assert fd.fdqp_describe(ctx, M, K, N).startswith("fdqp_prefill_stream_kernel")
+    y_ref, _ = case.reference()
+    ys = [torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda") for _ in range(4)]
+    for y in ys:                                       # back to back: a launch begins while the one before it ends
+        fd.fdqp_run(ctx, case.x_dev, case.W_dev, y, M, K, N)
+    torch.cuda.synchronize()
+    assert fd.fdqp_last_status(ctx) == 0
+    for y in ys:
+        assert np.array_equal(y.cpu().numpy().astype(np.float64), y_ref)
+
+
 @pytest.mark.parametrize("K,N,M,params", CUTS)
 def test_bf16_and_gated_stores(ctx, K, N, M, params):
     case = Case(K, N, M, seed=7500 + K + N + M)

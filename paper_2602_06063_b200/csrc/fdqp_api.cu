@@ -13,6 +13,7 @@
 #include "fdqp.h"
 #include "fdqp_format.h"
 #include "fdqp_plan.h"
+#include "fdqp_tensor_plan.h"
 
 namespace fdqp {
 cudaError_t gemv_launch(const GemvPlan& p, bool ahead, cudaStream_t stream);
@@ -44,19 +45,15 @@ using namespace fdqp;
 
 constexpr int kFlowKvClusterPositions = 2048;  // default of the "flowkv_cluster" parameter
 
-struct fdqp_ctx {
+struct fdqp_ctx : TensorSetup {
     int device = 0;
-    int sm_count = 0;
-    int smem_optin = 0;
     int64_t max_M = 0, max_K = 0, max_N = 0;
     float* ws_edge = nullptr;
     float* ws_full = nullptr;
-    float* pf_ws = nullptr;      // partial results of K-split tensor-core calls
+    float* pf_ws = nullptr;      // partial results of tensor-core calls (pf_ws_bytes)
     float* kv_ws = nullptr;      // decode attention: per (query head, split) partial results
     uint16_t* x_norm = nullptr;  // normalised activations of calls whose RMS normalisation cannot be fused (max_M x max_K)
     uint8_t* x_spread = nullptr; // small x copied with its rows further apart (see kSpreadBelowBytes)
-    size_t pf_ws_bytes = 0;
-    int st_clusters[3] = {0, 0, 0};  // streaming tensor-core kernel: clusters of 1, 2 and 4 pairs that fit the device at once
     int* pf_tickets = nullptr;   // arrival counters of tiles that pairs of SMs share
     int* tickets = nullptr;
     uint8_t* xq = nullptr;       // prepared activations of the call in flight
@@ -67,7 +64,7 @@ struct fdqp_ctx {
     int64_t launches = 0;
     std::string last_err;
     // overrides (-1 = automatic)
-    int64_t p_path = -1, p_ctas_per_sm = -1, p_cw = -1, p_stages = -1, p_split_k = -1, p_evict = -1, p_prep = -1, p_aligned = -1, p_bpw = -1, p_pair = -1, p_pf_split = -1;
+    int64_t p_ctas_per_sm = -1, p_cw = -1, p_stages = -1, p_split_k = -1, p_evict = -1, p_prep = -1, p_aligned = -1, p_bpw = -1;
     // fdqp_run_chain: partial rows of shared strips (2 per CTA and step), of whole strip-slices, arrival counters per
     // (step, strip), and the per-step completion counters followed by the exit counter
     float* chain_edge = nullptr;
@@ -76,11 +73,9 @@ struct fdqp_ctx {
     int* chain_done = nullptr;
     size_t chain_ticket_cap = 0;
     int64_t p_ahead = 1;  // kernels that read weights may begin, and read them, while the launch before them is finishing
-    int64_t p_st_tokens = -1, p_st_blocks = -1, p_st_cluster = -1;  // streaming tensor-core kernel: most tokens of a tile, blocks of a pair
     int64_t p_chain_launch = 1, p_chain_steps = kMaxChainSteps, p_chain_wide = 1, p_chain_dep = 0;
     int64_t p_flowkv_cluster = kFlowKvClusterPositions;  // ranges up to this many positions take the one-launch attention
     int64_t p_direct_y = 1;  // fdqp_run_host*: small results are stored straight into device-addressable host memory
-    int64_t p_atmem = 1;  // tensor-core tile kernel up to 128 tokens: keep the converted weights in tensor memory
     // Which kernels a call of these sizes takes, and their plan: a decode loop asks for the same few shapes again and again,
     // and the cost models take the host 1-2 us of a call's 8.  A function of the sizes and the parameters above alone
     // (fdqp_set_param empties it); nothing of a call's buffers is in it.
@@ -100,13 +95,9 @@ struct fdqp_ctx {
 namespace {
 
 constexpr int kMaxStages = 40;
-// Measured on B200: while all of x is smaller than 128 KB, the tensor-core kernels (every CTA re-reads the same few rows
-// of x by TMA at every k-step) run 1.45x slower; with the same rows placed further apart, so that they cover at least
-// 256 KB of addresses, the slow-down is gone.  Such an x is therefore copied into a spread-out staging buffer first.
-constexpr int64_t kSpreadBelowBytes = 128 << 10;
+// (x below kSpreadBelowBytes is copied so that its rows lie further apart)
 constexpr int64_t kSpreadToBytes = 256 << 10;
 constexpr size_t kSpreadBufBytes = (size_t)kSpreadToBytes + 256 * 128;  // row distance rounds up to 128 bytes, M <= 256 here
-constexpr int64_t kPrefillMinK = 256;          // shortest reduction the dispatch gives to the tensor-core kernels
 constexpr size_t kDirectHostBytes = 1u << 20;  // results up to this size go straight to addressable host memory
 constexpr int kKvMaxHeads = 64, kKvMaxSplits = 148, kKvMaxDim = 256;  // decode attention workspace
 constexpr size_t kPrefillWsCap = 128u << 20;  // bytes of partial results a context keeps for K-split tensor-core calls
@@ -143,217 +134,6 @@ fdqp_status check_shape(const fdqp_ctx* ctx, int64_t M, int64_t K, int64_t N) {
     if (M < 1 || K <= 0 || N <= 0 || (K % kGroup) != 0 || (N % kStripRows) != 0) return FDQP_ERR_SHAPE;
     if (M > ctx->max_M || K > ctx->max_K || N > ctx->max_N) return FDQP_ERR_SIZE;
     return FDQP_OK;
-}
-
-// More than 256 token rows: a pair of SMs works on a 256 x 512 tile (every converted weight serves 512 tokens).
-bool use_pair(const fdqp_ctx* ctx, int64_t M) { return ctx->p_pair >= 0 ? ctx->p_pair != 0 : M > 256; }
-
-// Time model of a tensor-core call cut into Z K slices (microseconds, without the launch and the optional spreading
-// copy; constants measured on B200).  A CTA (pair) costs about c per 64-wide k-step when its SM is full: c = 0.64 up to
-// 64 tokens rising to 0.72 at 128 (128-row tiles, two CTAs per SM), 0.78 (256-row tiles, one CTA per SM), 0.95 (two-SM
-// kernel).  The busiest SM runs n = ceil(CTAs / SMs) of them, two at a time where two fit; a CTA that has the SM to
-// itself runs its k-steps in about 0.7 of that time.  Z > 1 adds the second kernel (2-3 us on the stream: it overlaps the first one's tail) and the partial results:
-// written by the slices, read and summed by the second kernel.
-double prefill_time_model(const fdqp_ctx* ctx, int64_t M, int64_t K, int64_t N, int64_t Z) {
-    const bool pair = use_pair(ctx, M);
-    const bool small = !pair && M <= 128;
-    const int64_t tiles = pair ? ((N + 255) / 256) * ((M + 511) / 512)
-                               : (small ? (N + 127) / 128 : ((N + 255) / 256) * ((M + 255) / 256));
-    const int64_t units = pair ? ctx->sm_count / 2 : ctx->sm_count;
-    const int64_t n = (tiles * Z + units - 1) / units;
-    const double rounds = small ? (double)(n / 2) + ((n & 1) ? 0.7 : 0.0) : (double)n;
-    const double c = pair ? 0.95 : (M <= 64 ? 0.64 : (M <= 128 ? 0.64 + 0.08 * (double)(M - 64) / 64.0 : 0.78));
-    const int64_t kz = ((K + 63) / 64 + Z - 1) / Z;
-    double t = rounds * (double)kz * c;
-    if (Z > 1) t += 2.5 + (double)(2 * Z + 1) * (double)M * (double)N * 4.0 / 5.0e6;
-    return t;
-}
-
-// K slices of a tensor-core call: the count the time model likes best (a larger count has to win by 8 %), while every
-// slice keeps at least eight 64-wide k-steps and the partial results fit the context's workspace.  Few tiles (27B down:
-// 42 of 128 rows) get as many slices as fill the SMs once; a tile count just above a multiple of the slots (12B-like
-// K = 5376, N = 43008 at M = 32: 336 CTAs on 296 slots) gets the slices that even out the last round (85 -> 70 us).
-int prefill_slices(const fdqp_ctx* ctx, int64_t M, int64_t K, int64_t N) {
-    const int64_t ksteps = (K + 63) / 64;
-    int64_t zmax = kMaxSplit;
-    if (zmax > ksteps / 8) zmax = ksteps / 8;
-    const int64_t fit = (int64_t)(ctx->pf_ws_bytes / ((size_t)M * (size_t)N * 4));
-    if (zmax > fit) zmax = fit;
-    if (zmax < 1) zmax = 1;
-    if (ctx->p_pf_split > 0) return (int)(ctx->p_pf_split < zmax ? ctx->p_pf_split : zmax);
-    int64_t best = 1;
-    double t_best = prefill_time_model(ctx, M, K, N, 1);
-    for (int64_t Z = 2; Z <= zmax; ++Z) {
-        const double t = prefill_time_model(ctx, M, K, N, Z);
-        if (t < 0.95 * t_best) {
-            best = Z;
-            t_best = t;
-        }
-    }
-    return (int)best;
-}
-
-// Up to 128 tokens the one-SM kernel keeps the converted weights in tensor memory (mode 1, two CTAs per SM).  Up to 64
-// tokens a variant with half the accumulator columns, two weight stages and a four-deep weight prefetch (64 registers)
-// fits three CTAs per SM (mode 2): 6 % faster when the call has at least three CTAs per SM to run (LM head 181 -> 170 us),
-// slower when it has not (12B gate|up at M = 32: 44 -> 47 us), so the automatic choice asks for that many.
-int prefill_tmem_mode(const fdqp_ctx* ctx, int64_t M, int64_t K, int64_t N) {
-    if (ctx->p_atmem != 1) return (int)ctx->p_atmem;
-    if (M > 64) return 1;
-    const int64_t ctas = ((N + 127) / 128) * prefill_slices(ctx, M, K, N);
-    return ctas >= 3 * (int64_t)ctx->sm_count ? 2 : 1;
-}
-
-// ---- the streaming tensor-core kernel (fdqp_prefill_stream.cu) ----------------------------------------------------------
-// Time of one unit (a block of 256 k of a tile of 256 output features x n tokens) on a pair of SMs, us.  Measured on B200: up to
-// about 48 tokens the conversion of the weights sets the pace (K = 2560, N = 262144: 0.63 at 16 tokens, 0.70 at 48), then
-// conversion and x together (0.80 at 64, 1.05 at 128), then the MMAs (1.4 at 208, 1.7 at 256).
-double stream_unit_us(int n) { return n <= 128 ? 0.58 + 0.0035 * n : 1.03 + 0.0052 * (n - 128); }
-
-// What a launch loses when its CTAs have to wait for those of the launch before it, one to an SM: those of a launch on half of the
-// SMs or fewer find an SM, and have their barriers, tensor memory and first weights when the one before has ended.
-double stream_crowd_us(int64_t pairs) { return pairs <= 37 ? 0.0 : (pairs <= 50 ? 0.8 : 1.6); }
-
-// One way to cut a call: token tiles, and the range of units of a pair.
-struct StreamCut {
-    int64_t tok_tiles, per, pairs;  // per: units of the busiest pair
-    bool aligned;                   // ranges of whole tiles
-    int split;                      // pairs of a cluster that share a tile (1: ranges)
-    double us;
-};
-
-// per: units wanted for a pair; whole tiles when it is a multiple of nb.
-StreamCut stream_cut(const fdqp_ctx* ctx, int64_t M, int64_t nb, int64_t N, int64_t tok_tiles, int64_t per) {
-    const int64_t n = ((M + tok_tiles - 1) / tok_tiles + 15) / 16 * 16;
-    const int64_t units = (N + 255) / 256 * tok_tiles * nb;
-    StreamCut c{tok_tiles, per, (units + per - 1) / per, per % nb == 0, 1, 0.0};
-    c.us = (double)per * stream_unit_us((int)n);
-    // More than 128 tokens: one set of accumulators, so the pair's MMAs wait while a tile is read out (about 2 us).
-    const double reads = (double)((per + nb - 1) / nb);
-    if (n > 128) c.us += 2.0 * (reads > 1 ? reads - 1 : 0);
-    c.us += stream_crowd_us(c.pairs);
-    if (c.aligned) {
-        c.us += 0.004 * (double)n - 0.9;
-    } else {
-        // Tiles shared between pairs: partial sums out, a counter, and back in, by the piece; a range that begins in one tile and
-        // ends in another leaves two.  Measured at 37 tokens (us beyond 0.7 a unit and 3 for the launch): K = 10240, N = 2560
-        // 0.1 for 2 pieces, 2.1 for 4, 2.7 for 5, 4.6 for 7 or 8 with two to a range; K = 2560, N = 4096 1.1 for 2, 4.0 for 4 or 5.
-        const bool even = nb % per == 0;
-        const double pieces = (double)(even ? nb / per : nb / per + 2);
-        // At 200 tokens K = 2560, N = 4096 4.2 for 2 pieces, 10.5 for 4 or 5.
-        c.us += 0.2 + (0.12 + 0.0055 * (double)n) * pieces + (even ? 0.0 : 0.8) + 0.009 * (double)n;
-    }
-    return c;
-}
-
-// k-steps of x per stage: a block, so that the MMA issuer waits once per block; half of one where that would leave too few stages.
-int64_t stream_x_steps(int64_t n) { return n <= 96 ? 4 : 2; }
-int64_t stream_room(const fdqp_ctx* ctx) { return ctx->smem_optin - 1024 - kStBarBytes; }
-// Shared memory in which a CTA receives the sums of its cluster's other pairs: its strips' parts, 2 KB per 16 tokens and piece.
-int64_t stream_exchange_bytes(int64_t n, int split) {
-    return split == 1 ? 0 : 128 + 4 * (kStParts / split) * (int64_t)(split - 1) * 2048 * ((n + 16 * kStParts - 1) / (16 * kStParts));
-}
-
-// False: a launch parameter asks for one of the tile kernels, or the sizes are beyond this one's.
-bool plan_stream(const fdqp_ctx* ctx, int64_t M, int64_t K, int64_t N, int fmt, StreamParams* p, double* us) {
-    if (ctx->p_pair >= 0 || ctx->p_pf_split > 0 || !ctx->pf_ws) return false;
-    const int64_t nb = (K + kBlockK - 1) / kBlockK, sms = ctx->sm_count / 2;
-    const int64_t most = ctx->p_st_tokens > 0 ? ctx->p_st_tokens : kStMaxTokens;
-    const int64_t fewest = (M + most - 1) / most;
-    if (sms < 1 || (N + 255) / 256 * (fewest + 1) * nb > (int64_t)1 << 24) return false;
-    StreamCut best{};
-    for (int64_t tt = fewest; tt <= fewest + (M > 128 && ctx->p_st_tokens < 0 ? 1 : 0); ++tt) {
-        const int64_t n = ((M + tt - 1) / tt + 15) / 16 * 16, units = (N + 255) / 256 * tt * nb;
-        const int64_t least = (units + sms - 1) / sms, whole = ((N + 255) / 256 * tt + sms - 1) / sms * nb;  // fewest units, whole tiles
-        auto consider = [&](int64_t per) {
-            const StreamCut c = stream_cut(ctx, M, nb, N, tt, per);
-            if (!c.aligned && (size_t)(c.pairs * 2 * 8 * n * kStripRows * 4) > ctx->pf_ws_bytes) return;  // partial sums do not fit
-            if (!best.tok_tiles || c.us < best.us) best = c;
-        };
-        if (ctx->p_st_blocks > 0) {
-            consider(ctx->p_st_blocks > least ? ctx->p_st_blocks : least);
-            if (!best.tok_tiles) consider(whole);
-            continue;
-        }
-        // Few tiles: a cluster of two or four pairs for each, which add their sums through shared memory.
-        for (int i = 1; i < 3; ++i) {
-            const int64_t tiles = (N + 255) / 256 * tt, split = (int64_t)1 << i;
-            if (tiles * split > sms || tiles > ctx->st_clusters[i] || nb < split || tt > 1) continue;
-            // (beside the exchange: the fewest stages of packed weights, and two of x)
-            if (stream_exchange_bytes(n, (int)split) + kStMinW * 4 * (int64_t)fmt_block_bytes(fmt) + 2 * (stream_x_steps(n) * n * 64 + 16) > stream_room(ctx)) continue;
-            StreamCut c{tt, (nb + split - 1) / split, tiles * split, false, (int)split, 0.0};
-            // (measured as above: two pairs 0.1 at 48 tokens, 1.2 at 128, 2.6 when 32 clusters fill the device; four 1.4 and 3.3)
-            c.us = (double)c.per * stream_unit_us((int)n) + (split == 2 ? -0.2 : 0.5) + 0.008 * (double)n + 1.5 * stream_crowd_us(c.pairs);
-            if (ctx->p_st_cluster != 0 && (!best.tok_tiles || c.us < best.us)) best = c;
-        }
-        if (ctx->p_st_cluster == 1 && best.split > 1) continue;
-        consider(whole);
-        for (int64_t per = least; per < least + 64 && per < 2 * least + nb && per <= units; ++per) consider(per);
-    }
-    *us = best.us;
-    std::memset(p, 0, sizeof(*p));
-    p->M = (int)M;
-    p->K = (int)K;
-    p->N = (int)N;
-    p->nb = (int)nb;
-    p->tok_tiles = (int)best.tok_tiles;
-    p->n_inst = (int)(((M + best.tok_tiles - 1) / best.tok_tiles + 15) / 16 * 16);
-    p->tiles = (int)((N + 255) / 256 * best.tok_tiles);
-    const int64_t quanta = best.aligned ? p->tiles : (int64_t)p->tiles * nb;
-    p->quantum = (int)(best.aligned ? nb : 1);
-    p->pairs = (int)best.pairs;
-    p->split = best.split;
-    p->exchange_bytes = (uint32_t)stream_exchange_bytes(p->n_inst, p->split);
-    p->per_pair = (int)(quanta / best.pairs);
-    p->one_more = (int)(quanta % best.pairs);
-    // tensor memory: n_inst columns per set of accumulators, 128 per stage of converted weights
-    p->acc_sets = p->n_inst <= 128 ? 2 : 1;
-    p->a_stages = p->n_inst <= 64 ? 3 : 2;
-    // shared memory: x once and for all where it fits beside four blocks of weights, else rings of both
-    const int64_t x_steps = stream_x_steps(p->n_inst);
-    const int64_t w_stage = 4 * (int64_t)fmt_block_bytes(fmt), x_box = (int64_t)p->n_inst / 2 * 128, x_stage = x_steps * x_box + 16;
-    const int64_t room = stream_room(ctx) - (int64_t)p->exchange_bytes;
-    p->x_steps = (int)x_steps;
-    p->x_box_bytes = (uint32_t)x_box;
-    p->x_3d = K % 64 == 0;
-    p->x_stages = (int)((K + 64 * x_steps - 1) / (64 * x_steps));
-    p->x_resident = best.tok_tiles == 1 && x_steps == 4 && p->x_stages <= kStMaxX && p->x_stages * x_stage + kStMinW * w_stage <= room;
-    if (!p->x_resident) {
-        p->x_stages = (int)((room - kStMinW * w_stage) / x_stage);
-        if (p->x_stages > 12) p->x_stages = 12;
-    }
-    p->w_stages = (int)((room - p->x_stages * x_stage) / w_stage);
-    if (p->w_stages > kStMaxW) p->w_stages = kStMaxW;
-    p->smem_bytes = (uint32_t)(1024 + kStBarBytes + p->exchange_bytes + p->x_stages * x_stage + p->w_stages * w_stage);
-    p->ws = ctx->pf_ws;
-    p->tickets = ctx->pf_tickets;
-    p->status = ctx->status_dev;
-    return (p->x_resident || p->x_stages >= 2) && p->w_stages >= kStMinW;
-}
-
-// M >= 9: the tensor-core kernels, or the GEMV kernel eight token rows at a time -- whichever a small cost model
-// (microseconds, constants measured on B200) says is faster.
-//   GEMV: every chunk streams the whole matrix, at about 5.5 TB/s for 1-2 rows, 3.9 for 3-4, 3.2 for 5-8, plus ~8 us
-//   (back-to-back chunks of a small matrix: 2 x 15 us for 16 MB).
-//   Tensor-core kernels: prefill_time_model above.
-bool use_prefill(const fdqp_ctx* ctx, int64_t M, int64_t K, int64_t N, int fmt = kFmtQ4nx) {
-    if (M <= kMaxTokens || ctx->p_path == 2) return false;
-    if (ctx->p_path == 3) return true;
-    // The tensor-core kernels multiply by bf16-rounded weights (relative error up to 2^-8 per weight).  Against the
-    // acceptance bound 2e-3 * sum|x w| that is safe only where the K terms' rounding errors average out: with K = 32 two
-    // of 40,000 outputs were seen just outside it.  Short reductions therefore stay on the GEMV kernels (fp32 weights).
-    if (K < kPrefillMinK) return false;
-    const double mb = 0.625 * (double)K * (double)N / 1.0e6;  // packed weights, bytes per microsecond = TB/s * 1e6
-    const int64_t last = M % kMaxTokens;                       // rows of the ragged last chunk (0: none)
-    const double last_rate = last <= 2 ? 5.5 : (last <= 4 ? 3.9 : 3.2);
-    const double t_gemv = (double)(M / kMaxTokens) * (8.0 + mb / 3.2) + (last ? 8.0 + mb / last_rate : 0.0);
-    StreamParams stream;
-    double t_stream;
-    if (plan_stream(ctx, M, K, N, fmt, &stream, &t_stream)) return 3.5 + t_stream < t_gemv;
-    double t_tensor = 5.0 + prefill_time_model(ctx, M, K, N, prefill_slices(ctx, M, K, N));
-    if (prefill_tmem_mode(ctx, M, K, N) == 2) t_tensor *= 0.94;  // three CTAs per SM
-    if (M * K * 2 < kSpreadBelowBytes) t_tensor += 3.0;                                   // the spreading copy
-    return t_tensor < t_gemv;
 }
 
 // One way to lay a GEMV CTA out: warps, CTAs that share an SM, and the ring depth that leaves (0: does not fit).
@@ -559,6 +339,9 @@ fdqp_ctx::Dispatch dispatch_of(fdqp_ctx* ctx, int64_t M, int64_t K, int64_t N, i
     double us;
     if (d.tensor && plan_stream(ctx, M, K, N, fmt, &d.stream, &us)) {
         d.streamed = true;
+        d.stream.ws = ctx->pf_ws;
+        d.stream.tickets = ctx->pf_tickets;
+        d.stream.status = ctx->status_dev;
     } else if (d.tensor) {
         d.slices = prefill_slices(ctx, M, K, N);
         d.tmem_mode = prefill_tmem_mode(ctx, M, K, N);
@@ -656,7 +439,7 @@ extern "C" fdqp_status fdqp_create(fdqp_ctx** out, int device, int64_t max_M, in
         if ((e = chain_set_smem_limit(ctx->smem_optin))) { st = cuda_fail(nullptr, e, ""); break; }
         if ((e = gemv_set_smem_limit(ctx->smem_optin))) { st = cuda_fail(nullptr, e, ""); break; }
         if ((e = prefill_stream_set_smem_limit(ctx->smem_optin))) { st = cuda_fail(nullptr, e, ""); break; }
-        for (int i = 0; i < 3; ++i) ctx->st_clusters[i] = prefill_stream_max_clusters(2 << i, ctx->smem_optin);
+        for (int i = 0; i < 2; ++i) ctx->st_clusters[i] = prefill_stream_max_clusters(4 << i, ctx->smem_optin);
         if ((e = prefill_set_smem_limit())) { st = cuda_fail(nullptr, e, ""); break; }
         if ((e = cudaDeviceSynchronize())) { st = cuda_fail(nullptr, e, ""); break; }
     } while (false);

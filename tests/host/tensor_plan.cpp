@@ -1,0 +1,116 @@
+// The library's own plans of prefill-sized calls (fdqp_tensor_plan.h) over a grid of sizes: what the kernel relies on.
+#include <cstdio>
+#include <cstring>
+#include <map>
+#include <set>
+#include <vector>
+
+#include "fdqp_tensor_plan.h"
+
+using namespace fdqp;
+
+static long failed = 0;
+
+#define CHECK(what)                                                                       \
+    do {                                                                                  \
+        if (!(what) && ++failed <= 20) std::printf("M %lld K %lld N %lld: %s\n", (long long)M, (long long)K, (long long)N, #what); \
+    } while (0)
+
+static TensorSetup b200() {
+    TensorSetup s;
+    s.sm_count = 148;
+    s.smem_optin = 227 * 1024;
+    s.pf_ws_bytes = 128u << 20;
+    s.st_clusters[0] = 32;
+    s.st_clusters[1] = 14;
+    return s;
+}
+
+// Every unit of work in one range, memory and counters within their bounds, no slot of partial sums used twice.
+static void cut(const TensorSetup& setup, int64_t M, int64_t K, int64_t N, int fmt) {
+    StreamParams p;
+    double us;
+    const bool planned = plan_stream(&setup, M, K, N, fmt, &p, &us);
+    const int64_t most = setup.p_st_tokens > 0 ? setup.p_st_tokens : kStMaxTokens;
+    CHECK(planned || (N + 255) / 256 * ((M + most - 1) / most + 1) * ((K + 255) / 256) > 1 << 24);  // (more units than it counts)
+    if (failed || !planned) return;
+    CHECK(p.n_inst % 16 == 0 && p.n_inst <= kStMaxTokens && (int64_t)p.n_inst * p.tok_tiles >= M);
+    CHECK(p.nb == (K + 255) / 256 && p.tiles == (N + 255) / 256 * p.tok_tiles);
+    CHECK(p.acc_sets * p.n_inst + 128 * p.a_stages <= 512);
+    CHECK(p.a_stages >= 2 && p.a_stages <= 3 && p.w_stages >= kStMinW && p.w_stages <= kStMaxW);
+    CHECK(p.x_resident ? p.x_steps == 4 && p.x_stages == p.nb && p.tok_tiles == 1 : p.x_stages >= 2);
+    CHECK(p.x_stages <= kStMaxX);
+    CHECK((int64_t)p.smem_bytes <= setup.smem_optin);
+    CHECK((int64_t)p.smem_bytes == 1024 + kStBarBytes + p.exchange_bytes + (int64_t)p.x_stages * (p.x_steps * p.x_box_bytes + 16) + (int64_t)p.w_stages * 4 * fmt_block_bytes(fmt));
+    if (p.split > 1) {  // a cluster to a tile, a part of K to each of its pairs
+        CHECK(p.pairs == p.tiles * p.split && p.pairs <= setup.sm_count / 2 && p.tok_tiles == 1 && p.nb >= p.split && kStParts % p.split == 0);
+        return;
+    }
+    CHECK(p.pairs >= 1 && p.pairs <= setup.sm_count / 2 && p.per_pair >= 1 && (p.quantum == 1 || p.quantum == p.nb));
+    if (failed) return;
+    CHECK(st_range_begin(p, 0) == 0 && st_range_begin(p, p.pairs) == p.tiles * p.nb);
+    std::map<int, int> slots;
+    for (int r = 0; r < p.pairs; ++r) {
+        const int u0 = st_range_begin(p, r), u1 = st_range_begin(p, r + 1);
+        CHECK(u0 < u1);
+        for (int u = u0; u < u1;) {
+            const int tile = u / p.nb, end = u1 < (tile + 1) * p.nb ? u1 : (tile + 1) * p.nb;
+            if (u != tile * p.nb || end != (tile + 1) * p.nb) {
+                CHECK(p.quantum == 1 && st_owner(p, u) == r && st_owner(p, end - 1) == r);
+                CHECK(slots.emplace(2 * r + (u0 >= tile * p.nb ? 0 : 1), tile).second);
+            }
+            u = end;
+        }
+    }
+    if (slots.empty()) return;
+    CHECK((size_t)p.pairs * 2 * 8 * p.n_inst * kStripRows * 4 <= setup.pf_ws_bytes);
+    std::map<int, std::vector<int>> of_tile;
+    for (const auto& s : slots) of_tile[s.second].push_back(s.first);  // (in order of the slots, so of the pairs)
+    std::set<int> counters;
+    for (const auto& t : of_tile) {
+        const int p0 = st_owner(p, t.first * p.nb), p1 = st_owner(p, (t.first + 1) * p.nb - 1);
+        CHECK(p0 < p1 && counters.insert(p0).second);  // the first pair's counters serve one tile
+        // what the last arriver reads: the first pair's slot by where its range begins, the others' first ones
+        std::vector<int> read;
+        for (int r = p0; r <= p1; ++r) read.push_back(2 * r + (r == p0 && st_range_begin(p, p0) < t.first * p.nb ? 1 : 0));
+        CHECK(read == t.second);
+    }
+}
+
+static void cuts() {
+    const int64_t Ks[] = {32, 256, 288, 544, 768, 1152, 2560, 3840, 5376, 6912, 10240, 15360, 21504};
+    const int64_t Ns[] = {32, 64, 256, 288, 1024, 2560, 4096, 5376, 10240, 18944, 19200, 20480, 37888, 40960, 262144};
+    const int64_t Ms[] = {9, 16, 17, 37, 48, 64, 65, 96, 97, 112, 128, 129, 144, 200, 208, 256, 257, 300, 511, 512, 1000, 4096};
+    for (int64_t K : Ks)
+        for (int64_t N : Ns)
+            for (int64_t M : Ms) {
+                TensorSetup s = b200();
+                cut(s, M, K, N, kFmtQ4nx);
+                if (K % kBlockK == 0) cut(s, M, K, N, kFmtMxfp4);
+                for (int64_t blocks : {1, 2, 3, 7, 17, 1000000}) {
+                    s.p_st_blocks = blocks;
+                    cut(s, M, K, N, kFmtQ4nx);
+                }
+                s = b200();
+                for (int64_t tokens : {16, 112, 256}) {
+                    s.p_st_tokens = tokens;
+                    cut(s, M, K, N, kFmtQ4nx);
+                }
+                for (int cluster = 0; cluster < 2; ++cluster) {
+                    s = b200();
+                    s.p_st_cluster = cluster;
+                    cut(s, M, K, N, kFmtQ4nx);
+                }
+                s = b200();
+                s.pf_ws_bytes = 1 << 20;  // little room for partial sums
+                cut(s, M, K, N, kFmtQ4nx);
+            }
+}
+
+int main(int argc, char** argv) {
+    const char* what = argc > 1 ? argv[1] : "";
+    if (!std::strcmp(what, "cuts")) cuts();
+    else return 2;
+    std::printf("%ld wrong\n", failed);
+    return failed ? 1 : 0;
+}

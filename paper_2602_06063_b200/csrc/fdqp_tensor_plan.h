@@ -147,6 +147,7 @@ inline bool plan_stream(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N,
     StreamCut best{};
     for (int64_t tt = fewest; tt <= fewest + (M > 128 && ctx->p_st_tokens < 0 ? 1 : 0); ++tt) {
         const int64_t n = ((M + tt - 1) / tt + 15) / 16 * 16, units = (N + 255) / 256 * tt * nb;
+        if (tt > fewest && (tt - 1) * n >= M) continue;  // (rounded up to 16, a tile fewer holds every token)
         const int64_t least = (units + sms - 1) / sms, whole = ((N + 255) / 256 * tt + sms - 1) / sms * nb;  // fewest units, whole tiles
         auto consider = [&](int64_t per) {
             const StreamCut c = stream_cut(M, nb, N, tt, per);

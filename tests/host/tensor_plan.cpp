@@ -34,7 +34,7 @@ static void cut(const TensorSetup& setup, int64_t M, int64_t K, int64_t N, int f
     const int64_t most = setup.p_st_tokens > 0 ? setup.p_st_tokens : kStMaxTokens;
     CHECK(planned || (N + 255) / 256 * ((M + most - 1) / most + 1) * ((K + 255) / 256) > 1 << 24);  // (more units than it counts)
     if (failed || !planned) return;
-    CHECK(p.n_inst % 16 == 0 && p.n_inst <= kStMaxTokens && (int64_t)p.n_inst * p.tok_tiles >= M);
+    CHECK(p.n_inst % 16 == 0 && p.n_inst <= kStMaxTokens && (int64_t)p.n_inst * p.tok_tiles >= M && (int64_t)p.n_inst * (p.tok_tiles - 1) < M);
     CHECK(p.nb == (K + 255) / 256 && p.tiles == (N + 255) / 256 * p.tok_tiles);
     CHECK(p.acc_sets * p.n_inst + 128 * p.a_stages <= 512);
     CHECK(p.a_stages >= 2 && p.a_stages <= 3 && p.w_stages >= kStMinW && p.w_stages <= kStMaxW);

@@ -155,7 +155,8 @@ inline bool plan_stream(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N,
             if (!best.tok_tiles || c.us < best.us) best = c;
         };
         if (ctx->p_st_blocks > 0) {
-            consider(ctx->p_st_blocks > least ? ctx->p_st_blocks : least);
+            const int64_t wanted = ctx->p_st_blocks < units ? ctx->p_st_blocks : units;  // (more than there are: one pair)
+            consider(wanted > least ? wanted : least);
             if (!best.tok_tiles) consider(whole);
             continue;
         }

@@ -87,7 +87,7 @@ static void cuts() {
                 TensorSetup s = b200();
                 cut(s, M, K, N, kFmtQ4nx);
                 if (K % kBlockK == 0) cut(s, M, K, N, kFmtMxfp4);
-                for (int64_t blocks : {1, 2, 3, 7, 17, 1000000}) {
+                for (int64_t blocks : {(int64_t)1, (int64_t)2, (int64_t)3, (int64_t)7, (int64_t)17, (int64_t)1000000, INT64_MAX - 3, INT64_MAX}) {
                     s.p_st_blocks = blocks;
                     cut(s, M, K, N, kFmtQ4nx);
                 }

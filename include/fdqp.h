@@ -180,14 +180,16 @@ FDQP_API fdqp_status fdqp_destroy(fdqp_ctx* ctx);
  * Dispatch: M = 1 and 2..8 run the streaming GEMV kernels (weights fetched once
  * from HBM through a shared-memory ring, nibbles unpacked in registers, scale and
  * offset applied in fp32, split-K across CTAs reduced in a fixed order); M >= 9
- * runs either the dequantise-into-shared-memory tensor-core path (tcgen05,
- * accumulators in TMEM; a one-SM kernel up to 256 token rows, a two-SM kernel
- * above; K cut into slices when a shape has few output tiles) or the GEMV kernel
- * eight token rows at a time, whichever a small cost model expects to be faster
- * (GEMV chunks up to about 16-24 rows, or more when N is small).  Reductions
- * shorter than K = 256 always take the GEMV kernels: the tensor-core path
- * multiplies by bf16-rounded weights, whose rounding errors need a long K to
- * average out inside the acceptance bound.
+ * runs either the streaming tensor-core kernel (pairs of SMs that dequantise into
+ * tensor memory; tcgen05, accumulators in TMEM; ranges of the work or clusters of
+ * pairs where a shape has few output tiles) or the GEMV kernel eight token rows at
+ * a time.  The tensor-core path multiplies by weights rounded to bf16, so the line
+ * between them is one of accuracy: by a fixed rule on M, K and N, calls of few
+ * rows and few outputs take the GEMV kernels (with long K up to about 16 rows of
+ * 1024 outputs), and so do all reductions shorter than K = 256, whose rounding
+ * errors do not average out inside the acceptance bound.  For MXFP4, whose weights
+ * are bf16 numbers, a cost model takes the faster of the two.  "path"
+ * (fdqp_set_param) chooses either for every call.
  * How the GEMV kernels hold x.  M <= 2: each 32-group as 31-bit fixed point
  * relative to its largest exponent, in four signed byte planes that ride in the
  * columns of one integer tensor-core MMA per 16 rows -- exact for every bf16

@@ -213,11 +213,14 @@ inline bool plan_stream(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N,
     return (p->x_resident || p->x_stages >= 2) && p->w_stages >= kStMinW;
 }
 
-// M >= 9: the tensor-core kernels, or the GEMV kernel eight token rows at a time -- whichever a small cost model
-// (microseconds, constants measured on B200) says is faster.
+// M >= 9: the tensor-core kernels, or the GEMV kernel eight token rows at a time, by a small cost model (microseconds, constants
+// measured on B200).
 //   GEMV: every chunk streams the whole matrix, at about 5.5 TB/s for 1-2 rows, 3.9 for 3-4, 3.2 for 5-8, plus ~8 us
 //   (back-to-back chunks of a small matrix: 2 x 15 us for 16 MB).
-//   Tensor-core kernels: prefill_time_model above.
+//   Tensor-core kernels: where their rounding of the weights to bf16 costs accuracy (1.5e-3 of y against 1e-7), prefill_time_model:
+//   the line lies where the tile kernels overtake the GEMV chunks, and a faster tensor-core kernel does not move it, so that no call
+//   loses accuracy to one.  ("path" = 3 gives every call to them.)  MXFP4 weights are bf16 numbers: there the streaming kernel's own
+//   estimate decides.
 inline bool use_prefill(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N, int fmt = kFmtQ4nx) {
     if (M <= kMaxTokens || ctx->p_path == 2) return false;
     if (ctx->p_path == 3) return true;
@@ -231,7 +234,7 @@ inline bool use_prefill(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N,
     const double t_gemv = (double)(M / kMaxTokens) * (8.0 + mb / 3.2) + (last ? 8.0 + mb / last_rate : 0.0);
     StreamParams stream;
     double t_stream;
-    if (plan_stream(ctx, M, K, N, fmt, &stream, &t_stream)) return 3.5 + t_stream < t_gemv;
+    if (fmt == kFmtMxfp4 && plan_stream(ctx, M, K, N, fmt, &stream, &t_stream)) return 3.5 + t_stream < t_gemv;
     double t_tensor = 5.0 + prefill_time_model(ctx, M, K, N, prefill_slices(ctx, M, K, N));
     if (prefill_tmem_mode(ctx, M, K, N) == 2) t_tensor *= 0.94;  // three CTAs per SM
     if (M * K * 2 < kSpreadBelowBytes) t_tensor += 3.0;                                   // the spreading copy

@@ -107,9 +107,29 @@ static void cuts() {
             }
 }
 
+// Calls whose weights would lose accuracy in bf16 and that the GEMV kernels serve about as fast as the tile kernels; and such that
+// those serve faster.  MXFP4 weights lose nothing.
+static void routes() {
+    const struct { int64_t K, N, M; bool tensor, tensor_mx; } calls[] = {
+        {6912, 32, 9, false, true}, {6912, 256, 9, false, true}, {10240, 128, 12, false, true}, {15360, 1024, 9, false, true}, {15360, 1024, 10, false, true},
+        {21504, 1024, 9, false, true}, {21504, 1024, 16, false, true}, {21504, 1536, 9, false, true}, {21504, 1536, 10, false, true},
+        {2560, 2560, 9, true, true}, {10240, 2560, 9, true, true}, {21504, 1024, 32, true, true}, {6912, 1152, 24, true, true}, {256, 4096, 512, true, true}};
+    for (const auto& c : calls)
+        for (int fmt : {kFmtQ4nx, kFmtG64, kFmtG128, kFmtMxfp4}) {
+            const int64_t M = c.M, K = c.K, N = c.N;
+            TensorSetup s = b200();
+            CHECK(use_prefill(&s, M, K, N, fmt) == (fmt == kFmtMxfp4 ? c.tensor_mx : c.tensor));
+            s.p_path = 2;
+            CHECK(!use_prefill(&s, M, K, N, fmt));
+            s.p_path = 3;
+            CHECK(use_prefill(&s, M, K, N, fmt));
+        }
+}
+
 int main(int argc, char** argv) {
     const char* what = argc > 1 ? argv[1] : "";
     if (!std::strcmp(what, "cuts")) cuts();
+    else if (!std::strcmp(what, "routes")) routes();
     else return 2;
     std::printf("%ld wrong\n", failed);
     return failed ? 1 : 0;

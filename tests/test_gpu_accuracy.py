@@ -1,4 +1,5 @@
-"""Accuracy of the GEMV kernels at 3 to 8 tokens: no larger an error against 64 bits than per-group fp32 arithmetic has."""
+"""Accuracy of the GEMV kernels: at 3 to 8 tokens no larger an error against 64 bits than per-group fp32 arithmetic has; and which
+calls of nine and more rows they serve."""
 import math
 
 import pytest
@@ -79,3 +80,25 @@ def test_no_less_exact_than_per_group_sums(K, N, M, mx, slices):
     norm = exact.norm()
     got, allowed = float((y.double() - exact).norm() / norm), float((ref - exact).norm() / norm)
     assert got <= 1.02 * allowed, f"{got:.3e} against {allowed:.3e}"
+
+
+@pytest.mark.parametrize("K,N,M", [(6912, 256, 9), (21504, 1024, 9), (15360, 1024, 10)])
+def test_few_outputs_of_a_long_reduction_keep_fp32_weights(K, N, M):
+    """Nine and more rows that the GEMV kernels serve: fp32 sums of unrounded weights differ from 64 bits by 1e-7 .. 2e-7 (norm of the
+    difference over norm of y), weights rounded to bf16 by 1.5e-3.  The limit, 2e-6, lies ten times above the one."""
+    g = torch.Generator(device="cuda").manual_seed(K + M)
+    x = torch.randn((M, K), device="cuda", generator=g).to(torch.bfloat16)
+    codes, d, m = _weights(g, K, N, False)
+    W = _packed(codes, d, m, K, N)
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    ctx = fd.fdqp_create(0, M, K, N)
+    try:
+        assert "fdqp_gemv_kernel" in fd.fdqp_describe(ctx, M, K, N)
+        fd.fdqp_run(ctx, x, W, y, M, K, N)
+        torch.cuda.synchronize()
+        assert fd.fdqp_last_status(ctx) == 0
+    finally:
+        fd.fdqp_destroy(ctx)
+    w = codes.double() * d.double().repeat_interleave(32, dim=1) + m.double().repeat_interleave(32, dim=1)
+    exact = x.double() @ w.t()
+    assert float((y.double() - exact).norm() / exact.norm()) <= 2e-6

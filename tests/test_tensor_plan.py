@@ -28,3 +28,8 @@ def test_every_unit_once_within_the_bounds(program):
     """Streaming kernel: every unit of work in one pair's range, no slot of partial sums and no counter used twice, shared memory,
     tensor memory and workspace within their sizes."""
     check(program, "cuts")
+
+
+def test_calls_keep_fp32_weights(program):
+    """Which calls of nine and more rows go through the GEMV kernels, whose weights are not rounded to bf16."""
+    check(program, "routes")

@@ -469,7 +469,8 @@ FDQP_API const char* fdqp_status_string(fdqp_status s);
  *                   the splits of a KV head as a thread-block cluster merged through distributed shared memory;
  *                   longer ranges take the two-launch route (split kernel + merge kernel)
  *   "prefill_tokens" most token rows of a tile of the streaming tensor-core kernel (16 .. 256, a multiple of 16), which
- *                   takes every prefill-sized call unless "prefill_split_k" or "prefill_pair" is set
+ *                   takes every prefill-sized call unless "prefill_split_k", "prefill_pair" or, up to 128 token rows,
+ *                   "prefill_a_tmem" asks for the tile kernels
  *   "prefill_blocks" blocks of 256 k (of 256 output features x a token tile) that a pair of SMs works on in that kernel,
  *                   where the call has that many for each; a multiple of K / 256: whole tiles
  *   "prefill_cluster" that kernel may give a tile to a cluster of two or four pairs, which take a part of K each and add
@@ -481,10 +482,10 @@ FDQP_API const char* fdqp_status_string(fdqp_status s);
  *                   "prefill_split_k": two-SM kernel when M > 256
  *   "host_direct_y" fdqp_run_host*: 1 (default) = small x and y in device-addressable page-locked host memory are
  *                   read / written in place by the kernels, 0 = always through the staging buffers and copies
- *   "prefill_a_tmem" one-SM tensor-core tile kernel up to 128 token rows: 1 (default) = the converted weights are kept in
- *                   tensor memory and read from there by the MMAs (two CTAs per SM; up to 64 token rows three smaller
- *                   CTAs per SM when the call has that many to run), 2 = the three-CTA form whenever M <= 64,
- *                   0 = weights in shared memory; same results bit for bit
+ *   "prefill_a_tmem" one-SM tensor-core tile kernel up to 128 token rows: 1 (default; does not ask for that kernel) = the
+ *                   converted weights are kept in tensor memory and read from there by the MMAs (two CTAs per SM; up to
+ *                   64 token rows three smaller CTAs per SM when the call has that many to run), 2 = the three-CTA form
+ *                   whenever M <= 64, 0 = weights in shared memory; same results bit for bit
  * Unknown key or unusable value: FDQP_ERR_ARG.  Meant for benchmarks and tests. */
 FDQP_API fdqp_status fdqp_set_param(fdqp_ctx* ctx, const char* key, int64_t value);
 

@@ -891,16 +891,14 @@ extern "C" fdqp_status fdqp_describe(fdqp_ctx* ctx, int64_t M, int64_t K, int64_
         StreamParams sp;
         double us;
         if (plan_stream(ctx, M, K, N, kFmtQ4nx, &sp, &us)) {
-            const int n = std::snprintf(
+            std::snprintf(
                 buf, buf_bytes,
                 "fdqp_prefill_stream_kernel grid=%d cluster=%d block=768 smem=%u tile=256x%d token_tiles=%d cut=%s blocks_per_pair=%d..%d "
-                "accumulators=%d weight_blocks=%d+%d x_stages=%dx%d%s; by tiles: ",
+                "accumulators=%d weight_blocks=%d+%d x_stages=%dx%d%s",
                 2 * sp.pairs, 2 * sp.split, sp.smem_bytes, sp.n_inst, sp.tok_tiles, sp.split > 1 ? "clusters" : (sp.quantum > 1 || sp.nb == 1 ? "tiles" : "blocks"), sp.per_pair * sp.quantum,
                 (sp.per_pair + (sp.one_more != 0)) * sp.quantum, sp.acc_sets, sp.w_stages, sp.a_stages, sp.x_stages, sp.x_steps,
                 sp.x_resident ? " (all of x)" : "");
-            if (n < 0 || (size_t)n >= buf_bytes) return FDQP_OK;
-            buf += n;  // what "prefill_pair" and "prefill_split_k" would choose between
-            buf_bytes -= (size_t)n;
+            return FDQP_OK;
         }
         describe_tiles(ctx, M, K, N, buf, buf_bytes);
         return FDQP_OK;

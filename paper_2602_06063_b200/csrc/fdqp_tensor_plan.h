@@ -139,7 +139,7 @@ inline int64_t stream_exchange_bytes(int64_t n, int split) {
 
 // False: a launch parameter asks for one of the tile kernels, or the sizes are beyond this one's.
 inline bool plan_stream(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N, int fmt, StreamParams* p, double* us) {
-    if (ctx->p_pair >= 0 || ctx->p_pf_split > 0 || !ctx->pf_ws_bytes) return false;
+    if (ctx->p_pair >= 0 || ctx->p_pf_split > 0 || (ctx->p_atmem != 1 && M <= 128) || !ctx->pf_ws_bytes) return false;
     const int64_t nb = (K + kBlockK - 1) / kBlockK, sms = ctx->sm_count / 2;
     const int64_t most = ctx->p_st_tokens > 0 ? ctx->p_st_tokens : kStMaxTokens;
     const int64_t fewest = (M + most - 1) / most;

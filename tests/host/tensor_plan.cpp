@@ -126,10 +126,34 @@ static void routes() {
         }
 }
 
+// The parameters that ask for the tile kernels do so.
+static void tile_kernels() {
+    const int64_t K = 2560, N = 4096;
+    for (int64_t M : {9, 64, 128, 129, 512}) {
+        StreamParams p;
+        double us;
+        TensorSetup s = b200();
+        CHECK(plan_stream(&s, M, K, N, kFmtQ4nx, &p, &us));
+        for (int64_t v : {0, 1}) {
+            s.p_pair = v;
+            CHECK(!plan_stream(&s, M, K, N, kFmtQ4nx, &p, &us));
+        }
+        s = b200();
+        s.p_pf_split = 1;
+        CHECK(!plan_stream(&s, M, K, N, kFmtQ4nx, &p, &us));
+        for (int64_t v : {0, 2}) {  // (a form of the one-SM kernel up to 128 rows)
+            s = b200();
+            s.p_atmem = v;
+            CHECK(plan_stream(&s, M, K, N, kFmtQ4nx, &p, &us) == (M > 128));
+        }
+    }
+}
+
 int main(int argc, char** argv) {
     const char* what = argc > 1 ? argv[1] : "";
     if (!std::strcmp(what, "cuts")) cuts();
     else if (!std::strcmp(what, "routes")) routes();
+    else if (!std::strcmp(what, "tile_kernels")) tile_kernels();
     else return 2;
     std::printf("%ld wrong\n", failed);
     return failed ? 1 : 0;

@@ -71,11 +71,14 @@ CASES = [
     (4096, 4736, 8, {"strip_aligned": 0}),               # strips shared between CTAs (arrival counters)
     (10240, 320, 3, {"split_k": 4}),                     # K slices + sum kernel
     (1056, 320, 20, {"path": 2}),                        # GEMV eight rows at a time
-    (1056, 320, 40, {"path": 3}),                        # one-SM tensor-core kernel
+    (1056, 320, 40, {"path": 3}),                        # streaming tensor-core kernel
+    (1056, 320, 40, {"path": 3, "prefill_pair": 0}),     # one-SM tile kernel
+    (1056, 320, 200, {"path": 3, "prefill_pair": 0}),    # ... 256-row tiles
     (2048, 256, 64, {"path": 3, "prefill_split_k": 4}),  # ... with K slices + sum kernel
-    (1056, 320, 40, {"path": 3, "prefill_a_tmem": 2}),   # ... three CTAs per SM (up to 64 tokens)
+    (1056, 320, 40, {"path": 3, "prefill_pair": 0, "prefill_a_tmem": 2}),   # ... three CTAs per SM (up to 64 tokens)
     (2048, 256, 64, {"path": 3, "prefill_a_tmem": 2, "prefill_split_k": 4}),
-    (544, 1056, 300, {"path": 3}),                       # two-SM tensor-core kernel, ragged tokens
+    (544, 1056, 300, {"path": 3}),                       # streaming kernel, two token tiles
+    (544, 1056, 300, {"path": 3, "prefill_pair": 1}),    # two-SM tile kernel, ragged tokens
     (4096, 288, 512, {"path": 3, "prefill_split_k": 3}),
 ]
 
@@ -111,7 +114,7 @@ def test_geglu_epilogue_matches_oracle(fresh, K, N, M, params):
 
 
 @pytest.mark.parametrize("M,params", [(1, {}), (2, {}), (6, {"strip_aligned": 0}), (8, {"split_k": 2}), (24, {"path": 3}),
-                                      (300, {"path": 3})])
+                                      (300, {"path": 3}), (24, {"path": 3, "prefill_pair": 0}), (300, {"path": 3, "prefill_pair": 1})])
 def test_geglu_pairing_exact(fresh, M, params):
     # d = 2^-3, m = 1, x = 1: every y is an exact dyadic >= K, where gelu(g) = g in fp32 (tanh saturates), so the
     # output is exactly the bf16 of the exact product of rows r and r + 16 of each strip, as the oracle computes it

@@ -94,8 +94,8 @@ def test_projection_matches_oracle(ctx, fmt, K, N, M):
         assert_close(y[:, N - 256:], y_ref, a_ref, f"{NAMES[fmt]} K={K} N={N} M={M} tail")
 
 
-# Prefill-sized token counts: the tensor-core kernels (one-SM tile up to 256 tokens, SM pairs above; K slices when the
-# tiles are few), which dequantise the format into shared memory.
+# Prefill-sized token counts: the streaming tensor-core kernel, and the tile kernels (one-SM tile up to 256 tokens, SM pairs
+# above; K slices when the tiles are few), which dequantise the format into shared memory.
 PREFILL_SHAPES = [(2560, 4096, 64), (2560, 2048, 300), (3840, 1024, 130), (21504, 320, 40), (1280, 6912, 512), (512, 288, 17)]
 
 
@@ -106,19 +106,27 @@ def test_prefill_sized_projection_matches_oracle(ctx, fmt, K, N, M):
     c = FmtCase(fmt, K, N, M, 9000 + K + N + M + fmt, amp)
     fd.fdqp_set_param(ctx, "path", 3)       # the tensor-core kernels whatever the dispatch model would choose
     try:
-        y = c.run(ctx)
+        ys = {"streaming": c.run(ctx)}
+        fd.fdqp_set_param(ctx, "prefill_pair", 1 if M > 256 else 0)
+        ys["tiles"] = c.run(ctx)
         if M <= 64:                         # the three-CTAs-per-SM form of the one-SM kernel: the same bits
             fd.fdqp_set_param(ctx, "prefill_a_tmem", 2)
-            assert np.array_equal(c.run(ctx), y)
+            assert "three CTAs per SM" in fd.fdqp_describe(ctx, M, K, N)
+            assert np.array_equal(c.run(ctx), ys["tiles"])
+        if M <= 128:                        # weights in shared memory: the same bits
+            fd.fdqp_set_param(ctx, "prefill_a_tmem", 0)
+            assert np.array_equal(c.run(ctx), ys["tiles"])
     finally:
         fd.fdqp_set_param(ctx, "prefill_a_tmem", 1)
+        fd.fdqp_set_param(ctx, "prefill_pair", -1)
         fd.fdqp_set_param(ctx, "path", 0)
     n1 = min(N, 512)
-    y_ref, a_ref = c.reference(0, n1)
-    assert_close(y[:, :n1], y_ref, a_ref, f"{NAMES[fmt]} prefill K={K} N={N} M={M}")
-    if N > n1:
-        y_ref, a_ref = c.reference(N - 128, N)
-        assert_close(y[:, N - 128:], y_ref, a_ref, f"{NAMES[fmt]} prefill K={K} N={N} M={M} tail")
+    for kernel, y in ys.items():
+        y_ref, a_ref = c.reference(0, n1)
+        assert_close(y[:, :n1], y_ref, a_ref, f"{NAMES[fmt]} prefill, {kernel}, K={K} N={N} M={M}")
+        if N > n1:
+            y_ref, a_ref = c.reference(N - 128, N)
+            assert_close(y[:, N - 128:], y_ref, a_ref, f"{NAMES[fmt]} prefill, {kernel}, K={K} N={N} M={M} tail")
 
 
 def test_mxfp4_prefill_is_exact_on_exact_inputs(ctx):

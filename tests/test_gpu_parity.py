@@ -107,25 +107,29 @@ PREFILL = [(64, 32, 9), (1024, 512, 9), (1056, 320, 20), (2560, 1024, 100), (512
 
 @pytest.mark.parametrize("K,N,M", PREFILL)
 def test_prefill_tensor_path_matches_oracle(fresh, K, N, M):
-    # M >= 9: dequantise-into-shared-memory + tcgen05 path.  Ragged token tiles, a K that is not a multiple of
-    # the 64-wide pipeline step, N that is not a multiple of the 256-row tile, more than one token tile.
+    # M >= 9: dequantise + tcgen05.  Ragged token tiles, a K that is not a multiple of the 64-wide pipeline step, N that
+    # is not a multiple of the 256-row tile, more than one token tile.  By itself: the streaming kernel.
     case = Case(K, N, M, seed=2000 + K + N + M)
     fd.fdqp_set_param(fresh, "path", 3)
-    assert ("fdqp_prefill_pair_kernel" if M > 256 else "fdqp_prefill_kernel") in fd.fdqp_describe(fresh, M, K, N)
-    y = case.run(fresh)
+    assert fd.fdqp_describe(fresh, M, K, N).startswith("fdqp_prefill_stream_kernel")
     y_ref, a_ref = case.reference()
-    assert_close(y, y_ref, a_ref, f"prefill K={K} N={N} M={M}")
-    # the other tensor-core kernel (two-SM 256 x 512 tile <-> one-SM 256 x 256 tile) on the same inputs
-    fd.fdqp_set_param(fresh, "prefill_pair", 0 if M > 256 else 1)
-    assert ("fdqp_prefill_kernel" if M > 256 else "fdqp_prefill_pair_kernel") in fd.fdqp_describe(fresh, M, K, N)
-    assert_close(case.run(fresh), y_ref, a_ref, f"prefill (other tile) K={K} N={N} M={M}")
-    fd.fdqp_set_param(fresh, "prefill_pair", -1)
+    assert_close(case.run(fresh), y_ref, a_ref, f"prefill K={K} N={N} M={M}")
+    # the tile kernels (two-SM 256 x 512 tile, one-SM 256 x 256 or 128 x 128 tile) on the same inputs
+    fd.fdqp_set_param(fresh, "prefill_pair", 1)
+    assert fd.fdqp_describe(fresh, M, K, N).startswith("fdqp_prefill_pair_kernel")
+    assert_close(case.run(fresh), y_ref, a_ref, f"prefill (two-SM tile) K={K} N={N} M={M}")
+    fd.fdqp_set_param(fresh, "prefill_pair", 0)
+    assert fd.fdqp_describe(fresh, M, K, N).startswith("fdqp_prefill_kernel")
+    y = case.run(fresh)
+    assert_close(y, y_ref, a_ref, f"prefill (one-SM tile) K={K} N={N} M={M}")
     if M <= 128:
         # up to 128 token rows the converted weights live in tensor memory by default; in shared memory: the same bits
         assert "weights in TMEM" in fd.fdqp_describe(fresh, M, K, N)
         fd.fdqp_set_param(fresh, "prefill_a_tmem", 0)
         assert "weights in TMEM" not in fd.fdqp_describe(fresh, M, K, N)
         assert np.array_equal(case.run(fresh), y)
+        fd.fdqp_set_param(fresh, "prefill_pair", -1)        # (asked for by itself, this form still runs)
+        assert fd.fdqp_describe(fresh, M, K, N).startswith("fdqp_prefill_kernel") and "weights in TMEM" not in fd.fdqp_describe(fresh, M, K, N)
         fd.fdqp_set_param(fresh, "prefill_a_tmem", 1)
     # the same rows through the GEMV kernel, eight at a time: both are within the bound of the oracle
     fd.fdqp_set_param(fresh, "path", 2)
@@ -141,9 +145,9 @@ def test_prefill_three_ctas_per_sm_same_bits(fresh, K, N, M, Z):
     # oracle and bit for bit what the two-CTA form computes
     case = Case(K, N, M, seed=2500 + K + N + M)
     fd.fdqp_set_param(fresh, "path", 3)
-    if Z > 1:
-        fd.fdqp_set_param(fresh, "prefill_split_k", Z)
+    fd.fdqp_set_param(fresh, "prefill_split_k", Z)
     fd.fdqp_set_param(fresh, "prefill_a_tmem", 2)
+    assert fd.fdqp_describe(fresh, M, K, N).startswith("fdqp_prefill_kernel<128>")
     assert "three CTAs per SM" in fd.fdqp_describe(fresh, M, K, N)
     y3 = case.run(fresh)
     fd.fdqp_set_param(fresh, "prefill_a_tmem", 1)
@@ -160,6 +164,7 @@ def test_prefill_k_slices(fresh, K, N, M, Z):
     case = Case(K, N, M, seed=3000 + K + N + M)
     fd.fdqp_set_param(fresh, "path", 3)
     y_ref, a_ref = case.reference()
+    fd.fdqp_set_param(fresh, "prefill_pair", 1 if M > 256 else 0)
     auto = fd.fdqp_describe(fresh, M, K, N)
     if K >= 2048:                                               # long reductions over few tiles are split without being
         assert "split_k=" in auto and "split_k=1" not in auto  # asked (a short one is not worth the second kernel)

@@ -78,16 +78,22 @@ def test_gemma3_4b_lm_head_decode_and_prefill(ctx):
     assert np.all(np.isfinite(y))
 
 
-@pytest.mark.parametrize("M,form", [(48, "three CTAs per SM"), (128, "two CTAs per SM")])
-def test_gemma3_4b_lm_head_small_prefill_chunks(ctx, M, form):
-    # the one-SM forms of the tensor-core kernel at full size, in the configuration the dispatch picks by itself:
+@pytest.mark.parametrize("M,tiles,kernel,form", [(48, -1, "fdqp_prefill_stream_kernel", "cut=tiles"), (128, -1, "fdqp_prefill_stream_kernel", "cut=tiles"),
+                                                 (48, 0, "fdqp_prefill_kernel<128>", "three CTAs per SM"), (128, 0, "fdqp_prefill_kernel<128>", "two CTAs per SM")])
+def test_gemma3_4b_lm_head_small_prefill_chunks(ctx, M, tiles, kernel, form):
+    # the tensor-core kernel that the dispatch picks by itself, and the one-SM forms of the tile kernel, at full size:
     # 32 strips spread over N (first and last included), all M rows
     _, K, N, seed = synthgen.GEMMA3_4B_LM_HEAD
     w = synthgen.weights(seed, K, N)
     x = synthgen.activations(seed + 1, M, K)
     base = Case(K, N, M, seed, weights=w, x=x)
-    assert form in fd.fdqp_describe(ctx, M, K, N)
-    y = base.run(ctx)
+    fd.fdqp_set_param(ctx, "prefill_pair", tiles)
+    try:
+        shown = fd.fdqp_describe(ctx, M, K, N)
+        assert shown.startswith(kernel) and form in shown
+        y = base.run(ctx)
+    finally:
+        fd.fdqp_set_param(ctx, "prefill_pair", -1)
     assert np.all(np.isfinite(y))
     for s in np.unique(np.linspace(0, N // 32 - 1, 32).astype(np.int64)):
         n0 = int(s) * 32

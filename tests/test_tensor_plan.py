@@ -33,3 +33,7 @@ def test_every_unit_once_within_the_bounds(program):
 def test_calls_keep_fp32_weights(program):
     """Which calls of nine and more rows go through the GEMV kernels, whose weights are not rounded to bf16."""
     check(program, "routes")
+
+
+def test_parameters_select_the_tile_kernels(program):
+    check(program, "tile_kernels")

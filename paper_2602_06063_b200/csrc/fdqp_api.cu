@@ -406,9 +406,8 @@ extern "C" fdqp_status fdqp_create(fdqp_ctx** out, int device, int64_t max_M, in
             // K-split tensor-core calls (shapes with few output tiles): up to kMaxSplit partial results, capped
             const size_t want = (size_t)kMaxSplit * (size_t)max_M * (size_t)max_N * 4;
             ctx->pf_ws_bytes = want < kPrefillWsCap ? want : kPrefillWsCap;
-            // ... and the partial sums of tiles that pairs of SMs share: two per pair (39 MB for 256 and more tokens)
-            const size_t pairs = (size_t)ctx->sm_count / 2;
-            const size_t shared = pairs * 2 * 8 * (size_t)(max_M < kStMaxTokens ? (max_M + 15) / 16 * 16 : kStMaxTokens) * kStripRows * 4;
+            // ... and the partial sums of tiles that pairs of SMs share (39 MB for large matrices and 256 and more tokens)
+            const size_t pairs = (size_t)ctx->sm_count / 2, shared = stream_ws_bytes(ctx->sm_count, max_M, max_K, max_N);
             if (ctx->pf_ws_bytes < shared) ctx->pf_ws_bytes = shared;
             if ((e = cudaMalloc(&ctx->pf_tickets, pairs * kStTickets * sizeof(int)))) { st = cuda_fail(nullptr, e, ""); break; }
             if ((e = cudaMemset(ctx->pf_tickets, 0, pairs * kStTickets * sizeof(int)))) { st = cuda_fail(nullptr, e, ""); break; }

@@ -137,6 +137,22 @@ inline int64_t stream_exchange_bytes(int64_t n, int split) {
     return split == 1 ? 0 : 128 + 4 * (kStParts / split) * (int64_t)(split - 1) * 2048 * ((n + 16 * kStParts - 1) / (16 * kStParts));
 }
 
+// Partial sums of one pair of SMs: of the tile that its range begins in and of one that it shares with the next pair.
+inline size_t stream_slot_bytes(int64_t n) { return (size_t)2 * 8 * (size_t)n * kStripRows * 4; }
+// Workspace with which every call of a context has room for its partial sums: no more pairs work than there are units, and a call of
+// more token tiles has smaller ones.
+inline size_t stream_ws_bytes(int sm_count, int64_t max_M, int64_t max_K, int64_t max_N) {
+    const int64_t sms = sm_count / 2, units = (max_N + 255) / 256 * ((max_K + kBlockK - 1) / kBlockK);  // of one token tile
+    size_t most = 0;
+    for (int64_t tt = 1; tt <= (max_M + 15) / 16; ++tt) {
+        const int64_t rows = ((max_M + tt - 1) / tt + 15) / 16 * 16, n = rows < kStMaxTokens ? rows : kStMaxTokens;
+        const size_t bytes = (size_t)(units * tt < sms ? units * tt : sms) * stream_slot_bytes(n);
+        if (most < bytes) most = bytes;
+        if (units * tt >= sms) break;
+    }
+    return most;
+}
+
 // False: a launch parameter asks for one of the tile kernels, or the sizes are beyond this one's.
 inline bool plan_stream(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N, int fmt, StreamParams* p, double* us) {
     if (ctx->p_pair >= 0 || ctx->p_pf_split > 0 || (ctx->p_atmem != 1 && M <= 128) || !ctx->pf_ws_bytes) return false;
@@ -151,7 +167,7 @@ inline bool plan_stream(const TensorSetup* ctx, int64_t M, int64_t K, int64_t N,
         const int64_t least = (units + sms - 1) / sms, whole = ((N + 255) / 256 * tt + sms - 1) / sms * nb;  // fewest units, whole tiles
         auto consider = [&](int64_t per) {
             const StreamCut c = stream_cut(M, nb, N, tt, per);
-            if (!c.aligned && (size_t)(c.pairs * 2 * 8 * n * kStripRows * 4) > ctx->pf_ws_bytes) return;  // partial sums do not fit
+            if (!c.aligned && (size_t)c.pairs * stream_slot_bytes(n) > ctx->pf_ws_bytes) return;  // partial sums do not fit
             if (!best.tok_tiles || c.us < best.us) best = c;
         };
         if (ctx->p_st_blocks > 0) {

@@ -126,6 +126,32 @@ static void routes() {
         }
 }
 
+// A context's workspace holds the partial sums of each of its calls, and is no larger than its largest calls can need.
+static void workspaces() {
+    const int64_t contexts[][3] = {{9, 2560, 64}, {16, 1152, 6912}, {40, 10240, 32}, {48, 21504, 5376}, {128, 512, 256}, {200, 3840, 30720}, {300, 1056, 288},
+                                   {300, 256, 288}, {512, 21504, 262144}, {2000, 768, 1024}};
+    for (const auto& c : contexts) {
+        const int64_t M = c[0], K = c[1], N = c[2];
+        TensorSetup roomy = b200(), own = roomy;
+        own.pf_ws_bytes = stream_ws_bytes(roomy.sm_count, M, K, N);
+        // no more pairs than units of work at the most token tiles (16 rows each) or SMs, no larger tiles than the largest
+        const int64_t units = (N + 255) / 256 * ((K + 255) / 256) * ((M + 15) / 16), sms = roomy.sm_count / 2, rows = (M + 15) / 16 * 16;
+        CHECK(own.pf_ws_bytes <= (size_t)(units < sms ? units : sms) * 2 * 8 * 32 * 4 * (size_t)(rows < 256 ? rows : 256));
+        for (int64_t m = M; m > kMaxTokens; m = m * 7 / 8)
+            for (int64_t k = K; k > 0; k = k * 3 / 4 / 32 * 32)
+                for (int64_t n = N; n > 0; n = n * 2 / 3 / 32 * 32)
+                    for (int64_t tokens : {-1, 16, 64}) {
+                        roomy.p_st_tokens = own.p_st_tokens = tokens;
+                        StreamParams a, b;
+                        double us;
+                        const bool planned = plan_stream(&roomy, m, k, n, kFmtQ4nx, &a, &us);
+                        CHECK(plan_stream(&own, m, k, n, kFmtQ4nx, &b, &us) == planned && !std::memcmp(&a, &b, sizeof a));
+                    }
+    }
+    const int64_t M = 300, K = 1056, N = 288;  // ten units to a token tile
+    CHECK(stream_ws_bytes(148, M, K, N) <= 8 << 20);
+}
+
 // The parameters that ask for the tile kernels do so.
 static void tile_kernels() {
     const int64_t K = 2560, N = 4096;
@@ -154,6 +180,7 @@ int main(int argc, char** argv) {
     if (!std::strcmp(what, "cuts")) cuts();
     else if (!std::strcmp(what, "routes")) routes();
     else if (!std::strcmp(what, "tile_kernels")) tile_kernels();
+    else if (!std::strcmp(what, "workspaces")) workspaces();
     else return 2;
     std::printf("%ld wrong\n", failed);
     return failed ? 1 : 0;

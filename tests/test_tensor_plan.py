@@ -35,5 +35,9 @@ def test_calls_keep_fp32_weights(program):
     check(program, "routes")
 
 
+def test_workspace_of_a_context(program):
+    check(program, "workspaces")
+
+
 def test_parameters_select_the_tile_kernels(program):
     check(program, "tile_kernels")

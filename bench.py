@@ -3,8 +3,8 @@
 
 A step is one pass of the hot path over the largest single-GPU configuration: the Gemma3-4B tied LM head (K = 2560,
 N = 262144, 419 MB of packed Q4NX weights, seed 17) at decode M = 1 -- one fdqp_run call, one kernel launch.  The
-metric is the achieved bandwidth over the algorithmic bytes of the step (0.625*K*N + 2*M*K + 4*M*N).  Beside the
-headline the line carries one sub-object per BASELINE configuration and M (per-call median / min / p90 from CUDA-event
+metric is the achieved bandwidth over the algorithmic bytes of the step (0.625*K*N + 2*M*K + 4*M*N).  On stderr, before
+the headline's line, a JSON object with one sub-object per BASELINE configuration and M (per-call median / min / p90 from CUDA-event
 pairs, back-to-back mean from a graph replay of at least 60 ms, GB/s, fractions of the measured and the nominal peak,
 the launch plan and the clock samples of its own region), the Gemma3-4B layer as single calls and as chained launches,
 decode tokens/s (projections only: 34 layers + LM head), batched decode, the prefill tensor-core path, decode attention,
@@ -12,7 +12,7 @@ the format variants and the dequantisation engine.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Prints ONE JSON line.  With --impl reference the CPU oracle is timed instead, on the host cores.
+Prints ONE JSON line on stdout.  With --impl reference the CPU oracle is timed instead, on the host cores.
 """
 from __future__ import annotations
 
@@ -798,7 +798,7 @@ def run_ours(args, rank, local_rank, world):
                          "frac": step_bytes / head_us / 1e3 / peaks["hbm_gbs"],
                          # one ncu capture of this launch: dram__bytes_read.sum + dram__bytes_write.sum
                          "traffic": NCU_LM_HEAD_DRAM_BYTES, "peak_kind": peak_kind + " copy bandwidth",
-                         "kernel": "fdqp_gemv_kernel<16,1,4,false,Q4NX>", "launch_us": head_us},
+                         "kernel": "fdqp_gemv_kernel<16,1,false,Q4NX,1>", "launch_us": head_us},
             "cpu_baseline": cpu,
             "e2e": {"value": whole_job_gbs(step_bytes, e2e_steps, world, e2e_s * 1e3), "unit": "GB/s",
                     "h2d_bytes_per_step": 2 * M * hk, "d2h_bytes_per_step": 4 * M * hn, "ms_per_step": e2e_s / e2e_steps * 1e3,
@@ -806,7 +806,10 @@ def run_ours(args, rank, local_rank, world):
             "gpu_launches": kernels_per_step * timed_steps,
             "clocks": head_clocks or clocks_all,
         }
-        line.update(line_extra)
+        # the result line is kept short enough to be read whole from the end of a log: the tables go to stderr, before it
+        if line_extra:
+            line["decode_tokens_per_s"] = line_extra["decode_tokens_per_s"]
+            print(json.dumps(line_extra), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     fd.fdqp_destroy(ctx)
     if dist is not None:

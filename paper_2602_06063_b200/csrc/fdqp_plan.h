@@ -124,6 +124,16 @@ FDQP_HD inline int st_owner(const StreamParams& p, int unit) {
     return unit < big ? unit / (p.per_pair + 1) : p.one_more + (unit - big) / p.per_pair;
 }
 
+// Stages of x that a CTA loads for the units [u0, u1): a stage holds x_steps (2 or 4) of a block's four k-steps; a tile's last block
+// may have fewer of them.
+FDQP_HD inline int st_x_loads(int u0, int u1, int nb, int x_steps, int ksteps_last) {
+    const int n = u1 - u0;
+    return x_steps == 4 ? n : 2 * n - (ksteps_last <= 2 ? u1 / nb - u0 / nb : 0);
+}
+// Is the release of a ring's stage waited for: is there a load into it behind load i of all?  Other releases are not signalled: the
+// arrival goes to both CTAs of the pair, and what nobody waits for could reach one that has left, or its successor's barriers.
+FDQP_HD inline bool st_awaited(int i, int all, int stages) { return i + stages < all; }
+
 // The barrier (0, 1: of an accumulator set; kStAccLast) that tells that segment idx of a range, its idx-th part of a tile, is in the
 // accumulators, and the number of that barrier's phase.  A wait sees a phase's parity only, so its warp has to know the phase
 // before to be complete.  Warps that read every segment of a set do.  The last segment is read by the conversion warps, which

@@ -529,6 +529,8 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
             int kb = kb0, sx = p.x_resident ? per_block * kb : 0, sa = 0, b = 0;
             uint32_t pha = 0, phx = 0, phb = 0;
             bool first = true, ready = false;  // ready: the next block's first stages have been seen full
+            const int x_loads = p.x_resident ? 0 : st_x_loads(u0, u1, p.nb, p.x_steps, ksteps_last);
+            int ix = 0;
             for (int u = u0; u < u1 && ok; ++u) {
                 const bool wait_x = !p.x_resident || u - u0 < p.nb;  // (boxes that stay: full once and for all)
                 if (first && !(ok = warp_wait(acc_empty(b), phb ^ 1u, p.status))) break;
@@ -540,6 +542,7 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                 const int n = ksteps_of(kb);
                 const uint32_t d = (uint32_t)(b * p.n_inst), a = tmem_a + 128u * (uint32_t)sa, used_a = empty_a(sa);
                 const bool tile_end = kb + 1 == p.nb, done = tile_end || u + 1 == u1;  // this pair's part of the tile
+                const bool again_a = st_awaited(u - u0, u1 - u0, p.a_stages);
                 if (++sa == p.a_stages) {
                     sa = 0;
                     pha ^= 1u;
@@ -561,10 +564,11 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                                 for (int k4 = 0; k4 < 4; ++k4)
                                     umma2_bf16_ta(d, a + (uint32_t)(32 * j + 8 * k4), bdesc + (uint64_t)j * box + 2 * k4, idesc, first && j + k4 == 0 ? 0u : 1u);
                             }
-                        umma2_commit(used_a, pair_mask);
-                        if (!p.x_resident) umma2_commit(used_x, pair_mask);
+                        if (again_a) umma2_commit(used_a, pair_mask);
+                        if (st_awaited(ix, x_loads, p.x_stages)) umma2_commit(used_x, pair_mask);
                         if (done) umma2_commit(u + 1 == u1 ? acc_last : acc_full(b), pair_mask);
                     }
+                    ++ix;
                 } else {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -580,16 +584,17 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                                         umma2_bf16_ta(d, a + (uint32_t)(64 * h + 32 * j + 8 * k4), bdesc + (uint64_t)j * box + 2 * k4, idesc,
                                                       first && h + j + k4 == 0 ? 0u : 1u);
                                 }
-                            umma2_commit(empty_x(sx), pair_mask);
+                            if (st_awaited(ix, x_loads, p.x_stages)) umma2_commit(empty_x(sx), pair_mask);
                         }
                         __syncwarp();
+                        ++ix;
                         if (++sx == p.x_stages) {
                             sx = 0;
                             phx ^= 1u;
                         }
                     }
                     if (leader) {
-                        umma2_commit(used_a, pair_mask);
+                        if (again_a) umma2_commit(used_a, pair_mask);
                         if (done) umma2_commit(u + 1 == u1 ? acc_last : acc_full(b), pair_mask);
                     }
                 }

@@ -57,6 +57,23 @@ static void range(int nb, int kb0, int n, int sets, int a, int w) {
     }
 }
 
+// Every release of a stage that is signalled is waited for, and every one that is waited for is signalled: the loads of a range,
+// counted as the kernel makes them.
+static void releases(int nb, int kb0, int n, int ksteps_last, int x_steps, int stages) {
+    int loads = 0;
+    for (int u = kb0; u < kb0 + n; ++u)
+        for (int j = 0; j < (u % nb == nb - 1 ? ksteps_last : 4); j += x_steps) ++loads;
+    const int all = st_x_loads(kb0, kb0 + n, nb, x_steps, ksteps_last);
+    bool wrong = all != loads;
+    int signalled = 0;
+    for (int i = 0; i < loads; ++i) signalled += st_awaited(i, all, stages);
+    wrong |= signalled != (loads > stages ? loads - stages : 0);  // load i waits for the release of load i - stages
+    ++checked;
+    if (wrong && ++failed <= 20)
+        std::printf("releases: %d of %d loads (%d counted) signalled: K blocks %d (%d k-steps), first %d, range %d, %d stages\n", signalled, all, loads, nb,
+                    ksteps_last, kb0, n, stages);
+}
+
 int main() {
     const int forms[3][2] = {{2, 3}, {2, 2}, {1, 2}};  // accumulator sets, stages of converted weights
     for (int nb = 1; nb <= 6; ++nb)
@@ -64,6 +81,12 @@ int main() {
             for (int n = 1; n <= 39; ++n)
                 for (const auto& f : forms)
                     for (int w = kStMinW; w <= kStMaxW; ++w) range(nb, kb0, n, f[0], f[1], w);
+    for (int nb = 1; nb <= 5; ++nb)
+        for (int kb0 = 0; kb0 < nb; ++kb0)
+            for (int n = 1; n <= 24; ++n)
+                for (int ksteps_last = 1; ksteps_last <= 4; ++ksteps_last)
+                    for (int x_steps = 2; x_steps <= 4; x_steps += 2)
+                        for (int stages = 2; stages <= 12; ++stages) releases(nb, kb0, n, ksteps_last, x_steps, stages);
     std::printf("%ld states, %ld wrong\n", checked, failed);
     return failed ? 1 : 0;
 }

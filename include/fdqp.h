@@ -34,9 +34,10 @@
  * Dequantisation (Eq. 3):  w_hat = d * code + m, evaluated with d and m widened
  * exactly from bf16 and ONE rounding to fp32.  fdqp_dequant returns exactly that
  * value (or its round-to-nearest-even bf16).  fdqp_run accumulates in fp32 in an
- * unspecified but run-to-run reproducible order; for M >= 9 the weights pass
- * through bf16 before a tensor-core contraction.  Acceptance bound for y against
- * an fp64 evaluation: |y - y_ref| <= 2e-3 * sum_k |x*w_hat| + 1e-5.
+ * unspecified but run-to-run reproducible order; for M >= 9 the weights may pass
+ * through bf16 before a tensor-core contraction (d * code + m rounded to bf16 once,
+ * which is fdqp_dequant's bf16 value unless 0 < |m| < 2^-19 |d|).  Acceptance
+ * bound for y against an fp64 evaluation: |y - y_ref| <= 2e-3 * sum_k |x*w_hat| + 1e-5.
  * What the kernels guarantee for every finite input, and where the acceptance
  * bound follows from it:
  *   - M <= 8 (GEMV kernels): the activations enter the arithmetic EXACTLY (no

@@ -96,7 +96,7 @@ struct StreamParams {
     float* y;               // device, fp32 output [M][N] (epilogue kEpiNone)
     uint16_t* y16;          // device, bf16 output (other epilogues)
     float* ws;              // device, partial sums of tiles that pairs share: [pairs][2][8 strips][n_inst][32]
-    int* tickets;           // device, [pairs][8] arrival counters, zero between launches
+    int* tickets;           // device, [pairs][kStTickets] arrival counters, zero between launches
     int* status;            // host-mapped sticky status word
     int M, K, N, epi;
     int n_inst;             // tokens of a tile (a multiple of 16 up to 256)

@@ -1,14 +1,14 @@
 // Prefill-sized projection (M >= 9 token rows), the form every call takes unless a launch parameter asks for the tile kernels
 // of fdqp_prefill.cu: pairs of SMs that stay for the whole call and share its work to the block.
 //
-//   D[n][tok] = sum_k w16[k][n] * x[tok][k],   w16 = RNE_bf16( d * q + m )      (Eq. 3, then Eq. 14)
+//   D[n][tok] = sum_k w16[k][n] * x[tok][k],   w16 = RNE_bf16( d * q + m ), one rounding      (Eq. 3, then Eq. 14)
 //
 // Units of work are (tile of 256 output features x up to 256 tokens, block of 256 k); they lie tile by tile along one line that
 // is cut into one range per pair, at tile boundaries where that costs less than an exchange of partial sums.  Inside a CTA
 // (128 of the tile's rows) every part has its own warps and its own ring, so that nothing waits at a tile's end:
 //   warp 0   x boxes (TMA, 64 k x half of the tile's tokens; where the whole K of one token tile fits, loaded once and kept)
 //   warp 1   (CTA 0 of the pair) issues tcgen05.mma.cta_group::2, 256 rows x N tokens x 16 k
-//   warp 2   weights: whole packed blocks, cp.async.bulk into a ring
+//   warps 2, 3   weights: whole packed blocks, cp.async.bulk into a ring, two strips each
 //   warps 4..7   read finished accumulators and store y where there are two sets of them (up to 128 tokens); the last ones of a
 //                range, and all where there is one set, are read by the four conversion warps of a strip
 //   warps 8..23  convert: packed block -> bf16 pairs in registers -> tensor memory, where the MMA takes its A operand from;
@@ -87,10 +87,6 @@ __device__ __forceinline__ void tmem_st_16cols_async(uint32_t taddr, const uint3
         ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
           "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
-}
-__device__ __forceinline__ void keep_alive(const uint32_t (&r)[16]) {
-    asm volatile("" ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
-                 "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]));
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 

@@ -12,8 +12,9 @@ from gpu_common import ABS_TOL, MAX_K, MAX_M, REL_TOL, Case
 
 pytestmark = pytest.mark.gpu
 
-# up to eight rows 8192 values are held (M = 1: K too long for the projection to normalise itself), beyond that 4096
-ROWS = [(32, 3), (32, 9), (256, 9), (288, 4), (4096, 9), (4128, 9), (8192, 3), (8224, 8), (8224, 1), (21504, 2), (21504, 5), (21504, 9)]
+# up to eight rows 8192 values are held (M = 1: K too long for the projection to normalise itself), beyond that 4096; up to 2048 values
+# a single CTA takes a row whatever their number
+ROWS = [(1152, 2), (1152, 8), (2048, 2), (2048, 3), (2048, 8), (2080, 2), (2080, 3), (2080, 8), (32, 3), (32, 9), (256, 9), (288, 4), (4096, 9), (4128, 9), (8192, 3), (8224, 8), (8224, 1), (21504, 2), (21504, 5), (21504, 9)]
 
 
 @pytest.fixture(scope="module")

@@ -452,8 +452,8 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
         tmem_alloc2(tmem_slot, 512);
         tmem_relinquish2();
     } else if (warp == 4) {
-        if (lane == 12) mbar_init(acc_last, 1);
-        if (lane < 12) mbar_init(bars + 8u * (uint32_t)lane, lane < 4 ? 16u : (lane < 10 ? 1u : (p.acc_sets == 1 ? 8u * kStParts : 8u)));
+        if (lane < 13)
+            mbar_init(lane == 12 ? acc_last : bars + 8u * (uint32_t)lane, lane < 4 ? 16u : (lane < 10 || lane == 12 ? 1u : (p.acc_sets == 1 ? 8u * kStParts : 8u)));
         mbar_fence_init();
     } else if (warp == 6) {
         if (CLUSTER && lane < 16) mbar_init(exchange + 8u * (uint32_t)lane, (uint32_t)p.split - 1u);
@@ -525,8 +525,6 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
             int kb = kb0, sx = p.x_resident ? per_block * kb : 0, sa = 0, b = 0;
             uint32_t pha = 0, phx = 0, phb = 0;
             bool first = true, ready = false;  // ready: the next block's first stages have been seen full
-            const int x_loads = p.x_resident ? 0 : st_x_loads(u0, u1, p.nb, p.x_steps, ksteps_last);
-            int ix = 0;
             for (int u = u0; u < u1 && ok; ++u) {
                 const bool wait_x = !p.x_resident || u - u0 < p.nb;  // (boxes that stay: full once and for all)
                 if (first && !(ok = warp_wait(acc_empty(b), phb ^ 1u, p.status))) break;
@@ -538,7 +536,6 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                 const int n = ksteps_of(kb);
                 const uint32_t d = (uint32_t)(b * p.n_inst), a = tmem_a + 128u * (uint32_t)sa, used_a = empty_a(sa);
                 const bool tile_end = kb + 1 == p.nb, done = tile_end || u + 1 == u1;  // this pair's part of the tile
-                const bool again_a = st_awaited(u - u0, u1 - u0, p.a_stages);
                 if (++sa == p.a_stages) {
                     sa = 0;
                     pha ^= 1u;
@@ -560,11 +557,10 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                                 for (int k4 = 0; k4 < 4; ++k4)
                                     umma2_bf16_ta(d, a + (uint32_t)(32 * j + 8 * k4), bdesc + (uint64_t)j * box + 2 * k4, idesc, first && j + k4 == 0 ? 0u : 1u);
                             }
-                        if (again_a) umma2_commit(used_a, pair_mask);
-                        if (st_awaited(ix, x_loads, p.x_stages)) umma2_commit(used_x, pair_mask);
+                        umma2_commit(used_a, pair_mask);
+                        if (!p.x_resident) umma2_commit(used_x, pair_mask);
                         if (done) umma2_commit(u + 1 == u1 ? acc_last : acc_full(b), pair_mask);
                     }
-                    ++ix;
                 } else {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -580,17 +576,16 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
                                         umma2_bf16_ta(d, a + (uint32_t)(64 * h + 32 * j + 8 * k4), bdesc + (uint64_t)j * box + 2 * k4, idesc,
                                                       first && h + j + k4 == 0 ? 0u : 1u);
                                 }
-                            if (st_awaited(ix, x_loads, p.x_stages)) umma2_commit(empty_x(sx), pair_mask);
+                            umma2_commit(empty_x(sx), pair_mask);
                         }
                         __syncwarp();
-                        ++ix;
                         if (++sx == p.x_stages) {
                             sx = 0;
                             phx ^= 1u;
                         }
                     }
                     if (leader) {
-                        if (again_a) umma2_commit(used_a, pair_mask);
+                        umma2_commit(used_a, pair_mask);
                         if (done) umma2_commit(u + 1 == u1 ? acc_last : acc_full(b), pair_mask);
                     }
                 }
@@ -609,12 +604,21 @@ __global__ void __launch_bounds__(kStThreads, 1) fdqp_prefill_stream_kernel(cons
         int s = w_first == p.w_stages ? 0 : w_first;
         uint32_t ph = 0;  // (the first round is under way)
         for (int u = u0 + w_first; u < u1; ++u) {
-            if (!warp_wait(empty_w(s), ph, p.status)) break;
+            if (!(ok = warp_wait(empty_w(s), ph, p.status))) break;
             load_blocks(s);
             if (++s == p.w_stages) {
                 s = 0;
                 ph ^= 1u;
             }
+        }
+        // The last release of every stage of converted weights and of x has arrived (beside the read-out of the last sums; a lane a
+        // barrier).
+        if (warp == 2 && ok && warp_wait(acc_last, 0, p.status)) {
+            const int x_loads = p.x_resident ? 0 : st_x_loads(u0, u1, p.nb, p.x_steps, ksteps_last);
+            const bool of_a = lane < 4;
+            const int s = of_a ? lane : lane - 4, stages = of_a ? p.a_stages : p.x_stages;
+            const int uses = s < stages ? st_stage_uses(s, of_a ? u1 - u0 : x_loads, stages) : 0;
+            if (uses) mbar_wait(of_a ? empty_a(s) : empty_x(s), (uint32_t)(uses - 1) & 1u, p.status);
         }
     } else {
         // =============================== conversion; accumulators -> y =======================================

@@ -57,21 +57,22 @@ static void range(int nb, int kb0, int n, int sets, int a, int w) {
     }
 }
 
-// Every release of a stage that is signalled is waited for, and every one that is waited for is signalled: the loads of a range,
-// counted as the kernel makes them.
+// The last release of every stage, for which the kernel waits before it ends: the loads of a range and the uses of each stage, counted as
+// the kernel makes them.
 static void releases(int nb, int kb0, int n, int ksteps_last, int x_steps, int stages) {
     int loads = 0;
     for (int u = kb0; u < kb0 + n; ++u)
         for (int j = 0; j < (u % nb == nb - 1 ? ksteps_last : 4); j += x_steps) ++loads;
     const int all = st_x_loads(kb0, kb0 + n, nb, x_steps, ksteps_last);
     bool wrong = all != loads;
-    int signalled = 0;
-    for (int i = 0; i < loads; ++i) signalled += st_awaited(i, all, stages);
-    wrong |= signalled != (loads > stages ? loads - stages : 0);  // load i waits for the release of load i - stages
+    for (int s = 0; s < stages; ++s) {
+        int uses = 0;
+        for (int i = s; i < loads; i += stages) ++uses;
+        wrong |= st_stage_uses(s, all, stages) != uses;
+    }
     ++checked;
     if (wrong && ++failed <= 20)
-        std::printf("releases: %d of %d loads (%d counted) signalled: K blocks %d (%d k-steps), first %d, range %d, %d stages\n", signalled, all, loads, nb,
-                    ksteps_last, kb0, n, stages);
+        std::printf("releases: %d loads, %d counted: K blocks %d (%d k-steps), first %d, range %d, %d stages\n", all, loads, nb, ksteps_last, kb0, n, stages);
 }
 
 int main() {
